@@ -818,6 +818,31 @@ int dbm_step(dbm_t *h, int64_t nsteps, void *stream)
 }  // extern "C"
 
 template <typename real>
+static cudaError_t launch_noneq_as(dbm_t *h, double *d_out, cudaStream_t s)
+{
+    const dbm_params &p = h->p;
+    MomArgs<real> A;
+    std::memset(&A, 0, sizeof(A));
+    A.f = reinterpret_cast<const real *>(h->buf + h->L.f[h->cur]);
+    A.out = d_out;
+    A.plane = h->plane;
+    A.nr = p.nr;
+    A.ntheta = p.ntheta;
+    A.ld = h->ld;
+    A.th_over_pi = theta_span(p) / PI / p.ntheta;
+    for (int k = 0; k < 4; ++k) {
+        A.v[k] = p.v[k];
+        A.v2[k] = p.v[k] * p.v[k];
+        A.v3[k] = A.v2[k] * p.v[k];
+        A.v4[k] = A.v2[k] * A.v2[k];
+    }
+    A.m0 = 0;
+    A.m1 = p.ntheta;
+    const long long blocks = ((long long)p.nr * p.ntheta + 255) / 256;
+    return launch_noneq<real>(A, (int)std::min<long long>(blocks, 1 << 20), s);
+}
+
+template <typename real>
 static cudaError_t launch_moments_as(dbm_t *h, double *d_out, double *partials, int grid, cudaStream_t s,
                                      int m0, int m1)
 {
@@ -837,8 +862,6 @@ static cudaError_t launch_moments_as(dbm_t *h, double *d_out, double *partials, 
     A.r_in = p.r_in;
     A.dr = (p.r_out - p.r_in) / p.nr;
     A.dtheta = theta_span(p) / p.ntheta;
-    A.th_over_pi = theta_span(p) / PI / p.ntheta;
-    std::memcpy(A.v, p.v, sizeof(A.v));
     for (int k = 0; k < 4; ++k) {
         A.vr[k] = (real)p.v[k];
         A.v2r[k] = (real)(p.v[k] * p.v[k]);
@@ -883,39 +906,8 @@ static int launch_moments_into(dbm_t *h, double *d_out, cudaStream_t s)
 
 static int launch_noneq_into(dbm_t *h, double *d_out, cudaStream_t s)
 {
-    const dbm_params &p = h->p;
-    const long long N = (long long)p.nr * p.ntheta;
-    const int grid = (int)std::min<long long>((N + 255) / 256, 4096);
-    cudaError_t e;
-    if (p.precision == DBM_FP64) {
-        MomArgs<double> A;
-        std::memset(&A, 0, sizeof(A));
-        A.f = reinterpret_cast<const double *>(h->buf + h->L.f[h->cur]);
-        A.out = d_out;
-        A.plane = h->plane;
-        A.nr = p.nr;
-        A.ntheta = p.ntheta;
-        A.ld = h->ld;
-        A.th_over_pi = theta_span(p) / PI / p.ntheta;
-        std::memcpy(A.v, p.v, sizeof(A.v));
-        A.m0 = 0;
-        A.m1 = p.ntheta;
-        e = launch_noneq<double>(A, grid, s);
-    } else {
-        MomArgs<float> A;
-        std::memset(&A, 0, sizeof(A));
-        A.f = reinterpret_cast<const float *>(h->buf + h->L.f[h->cur]);
-        A.out = d_out;
-        A.plane = h->plane;
-        A.nr = p.nr;
-        A.ntheta = p.ntheta;
-        A.ld = h->ld;
-        A.th_over_pi = theta_span(p) / PI / p.ntheta;
-        std::memcpy(A.v, p.v, sizeof(A.v));
-        A.m0 = 0;
-        A.m1 = p.ntheta;
-        e = launch_noneq<float>(A, grid, s);
-    }
+    const cudaError_t e = h->p.precision == DBM_FP64 ? launch_noneq_as<double>(h, d_out, s)
+                                                     : launch_noneq_as<float>(h, d_out, s);
     if (e != cudaSuccess) return cuda_fail(e, "noneq kernel launch");
     return DBM_OK;
 }

@@ -1237,19 +1237,6 @@ static __global__ void rcp_selftest_kernel(const float *x, float *approx, float 
 // all finite): a block that finds a bad one sets *bad, which the host reports
 // as DBM_EINVAL (the state is then undefined).
 // ---------------------------------------------------------------------------
-// Cartesian direction cosines of the 8 directions i pi / 4 (FP64 kernels).
-__device__ __forceinline__ void cart_dirs(double (&cx)[8], double (&cy)[8])
-{
-    const double H = 0.70710678118654752440;
-    const double c[8] = {1.0, H, 0.0, -H, -1.0, -H, 0.0, H};
-    const double sn[8] = {0.0, H, 1.0, H, 0.0, -H, -1.0, -H};
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        cx[i] = c[i];
-        cy[i] = sn[i];
-    }
-}
-
 template <typename real>
 struct InitArgs {
     const double *fields;
@@ -1322,13 +1309,56 @@ __global__ void __launch_bounds__(256) init_kernel(const InitArgs<real> A)
 }
 
 // ---------------------------------------------------------------------------
+// FP64 diagnostics.  GB300 issues one FP64 warp instruction per 19 cycles and
+// SM (one per 64 cycles and SM quarter), conversions to and from FP64
+// included, so these kernels cost what they count in FP64 instructions, tens
+// of times their memory time.  A ring's eight f are therefore reduced first,
+// by additions alone, to the harmonics its moments need (the velocities of a
+// ring are v_k (cos i pi/4, sin i pi/4)), and all moments are taken from the
+// few ring harmonics.
+// ---------------------------------------------------------------------------
+// f widened to FP64.  Normal floats by shifting their bits: three integer
+// instructions in place of a conversion at the FP64 rate.
+__device__ __forceinline__ double widen(double x) { return x; }
+__device__ __forceinline__ double widen(float x)
+{
+    const uint32_t b = __float_as_uint(x), e = b & 0x7f800000u;
+    if (e == 0u || e == 0x7f800000u) return (double)x;  // zero, subnormal, infinity, NaN
+    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
+}
+
+// Harmonics of a ring's f: s0 = sum g, (c1, s1) = sum g (cos, sin)(phi),
+// (c2, s2) of 2 phi, (c3, s3) of 3 phi, phi = i pi / 4.
+struct RingHarmonics {
+    double s0, c1, s1, c2, s2, c3, s3;
+};
+__device__ __forceinline__ RingHarmonics ring_harmonics(const double (&g)[8])
+{
+    const double H = 0.70710678118654752440;
+    const double p0 = g[0] + g[4], p1 = g[1] + g[5], p2 = g[2] + g[6], p3 = g[3] + g[7];
+    const double d0 = g[0] - g[4], d1 = g[1] - g[5], d2 = g[2] - g[6], d3 = g[3] - g[7];
+    const double a = d1 - d3, b = d1 + d3;
+    RingHarmonics r;
+    r.s0 = (p0 + p2) + (p1 + p3);
+    r.c2 = p0 - p2;
+    r.s2 = p1 - p3;
+    r.c1 = fma(H, a, d0);
+    r.c3 = fma(-H, a, d0);
+    r.s1 = fma(H, b, d2);
+    r.s3 = fma(H, b, -d2);
+    return r;
+}
+
+// ---------------------------------------------------------------------------
 // Moments (Sec. II.B) from f, plus per-block partial sums of the
 // area-weighted totals {mass, momentum x, momentum y, energy}, summed in FP64
-// across sites.  FP64 states: every site in FP64.  FP32 states: each site's
-// rho, rho u and sum f v^2 in FP32, ring by ring exactly as the step computes
-// them (ring_moments), u and T from those in FP32; the outputs are those
-// values widened to double (the FP32 state itself carries ~6e-8 relative
-// rounding per value, so FP64 per-site arithmetic would add no accuracy).
+// across sites.  Each site's rho, rho u and sum f v^2 are taken in the state's
+// precision ring by ring exactly as the step computes them (ring_moments), u
+// and T from those; FP32 values are widened to double (the FP32 state itself
+// carries ~6e-8 relative rounding per value, so FP64 per-site arithmetic would
+// add no accuracy).  The FP64 kernel is bound by its FP64 instructions: about
+// 110 per site this way, 369 with per-velocity sums, a second pass for T and
+// the row's angle evaluated at every site.
 // out: [5][ntheta][nr] doubles; partials: [gridDim.x][4] (scratch).
 // ---------------------------------------------------------------------------
 template <typename real>
@@ -1338,13 +1368,13 @@ struct MomArgs {
     double *out;
     double *partials;
     int *status;
-    const real *rowtab;  // [ntheta][16] (FP32 moments)
+    const real *rowtab;  // [ntheta][16] (moments)
     long long plane;
     int nr, ntheta, ld;
     double r_in, dr, dtheta;
     double th_over_pi;  // theta_m / pi per row
-    double v[4];
-    real vr[4], v2r[4];  // ring speeds and squares in real (FP32 moments)
+    double v[4], v2[4], v3[4], v4[4];  // ring speeds and their powers
+    real vr[4], v2r[4];  // ring speeds and squares in real (moments)
     int m0, m1;          // theta rows [m0, m1) of this launch
 };
 
@@ -1393,33 +1423,21 @@ __global__ void __launch_bounds__(256) moments_kernel(const MomArgs<real> A)
         acc[2] *= wa;
         acc[3] *= 0.5 * wa;
     } else {
-        double cx[8], cy[8];
-        cart_dirs(cx, cy);
+        const double wa = A.dr * A.dtheta;
         for (long long s = (long long)A.m0 * A.nr + blockIdx.x * (long long)blockDim.x + threadIdx.x;
              s < (long long)A.m1 * A.nr; s += (long long)gridDim.x * blockDim.x) {
             const int m = (int)(s / A.nr), j = (int)(s - (long long)m * A.nr);
             const real *fp = A.f + (long long)m * A.ld + j;
-            double fv[NV];
-            for (int q = 0; q < NV; ++q) fv[q] = (double)fp[(long long)q * A.plane];
-            double rho = fv[0], jx = 0.0, jy = 0.0;
-            for (int k = 0; k < 4; ++k)
-                for (int i = 0; i < 8; ++i) {
-                    const double fq = fv[1 + 8 * k + i];
-                    rho += fq;
-                    jx += fq * A.v[k] * cx[i];
-                    jy += fq * A.v[k] * cy[i];
-                }
-            const double ux = jx / rho, uy = jy / rho;
-            double e = 0.5 * fv[0] * (ux * ux + uy * uy);
-            for (int k = 0; k < 4; ++k)
-                for (int i = 0; i < 8; ++i) {
-                    const double dx = A.v[k] * cx[i] - ux, dy = A.v[k] * cy[i] - uy;
-                    e += 0.5 * fv[1 + 8 * k + i] * (dx * dx + dy * dy);
-                }
-            const double T = e / rho;
-            double sth, cth;
-            sincospi(A.th_over_pi * m, &sth, &cth);
-            const double ur = ux * cth + uy * sth, uth = -ux * sth + uy * cth;
+            real fv[NV];
+#pragma unroll
+            for (int q = 0; q < NV; ++q) fv[q] = fp[(long long)q * A.plane];
+            real rho, jx, jy, e2;
+            ring_moments<real>(fv, A.vr, A.v2r, rho, jx, jy, e2);
+            const double inv_rho = 1.0 / rho;
+            const double ux = jx * inv_rho, uy = jy * inv_rho;
+            const double T = 0.5 * fma(e2, inv_rho, -fma(ux, ux, uy * uy));
+            const double cth = A.rowtab[(long long)m * 16], sth = -A.rowtab[(long long)m * 16 + 8];
+            const double ur = fma(ux, cth, uy * sth), uth = fma(uy, cth, -(ux * sth));
             const double lam = LamStore<real>::to_lambda((double)A.lam[(long long)m * A.ld + j]);
             if (A.out) {
                 A.out[s] = rho;
@@ -1429,12 +1447,16 @@ __global__ void __launch_bounds__(256) moments_kernel(const MomArgs<real> A)
                 A.out[4 * N + s] = lam;
             }
             bad |= !isfinite(rho) || !isfinite(ur) || !isfinite(uth) || !isfinite(T) || !isfinite(lam);
-            const double w = (A.r_in + (j + 0.5) * A.dr) * A.dr * A.dtheta;
-            acc[0] += rho * w;
-            acc[1] += rho * ux * w;
-            acc[2] += rho * uy * w;
-            acc[3] += (rho * T + 0.5 * rho * (ux * ux + uy * uy)) * w;
+            const double r = A.r_in + (j + 0.5) * A.dr;  // weight r dr dtheta: dr dtheta applied per block
+            acc[0] = fma(rho, r, acc[0]);
+            acc[1] = fma(jx, r, acc[1]);
+            acc[2] = fma(jy, r, acc[2]);
+            acc[3] = fma(e2, r, acc[3]);  // rho T + rho u^2 / 2 = (1/2) sum f v^2 for D = 2
         }
+        acc[0] *= wa;
+        acc[1] *= wa;
+        acc[2] *= wa;
+        acc[3] *= 0.5 * wa;
     }
     if (bad) atomicOr(A.status, ST_NONFINITE);
     // deterministic block reduction: warp shuffles, then warp 0 over the warps
@@ -1463,54 +1485,105 @@ __global__ void __launch_bounds__(256) moments_kernel(const MomArgs<real> A)
 // Maxwellian's (M*_2 = rho T I, M*_3 = M*_{3,1} = 0, M*_{4,2} = 2 rho T^2 I for
 // D = 2), so only f's moments are summed.  out: [12][ntheta][nr] doubles in the
 // order rr, rth, thth | rrr, rrth, rthth, ththth | r, th | rr, rth, thth.
+// Raw moments of order up to four from the ring harmonics, turned into the
+// site's polar frame harmonic by harmonic (an n-th harmonic turns by n theta),
+// then made central with u.  About 240 FP64 instructions per site where the
+// 33 x 12 direct sums took 1180.  The row's angles are evaluated once per
+// block and row.
 template <typename real>
 __global__ void __launch_bounds__(256) noneq_kernel(const MomArgs<real> A)
 {
+    __shared__ double trig[256][6];  // cos, sin of theta, 2 theta, 3 theta of the block's rows
     const long long N = (long long)A.nr * A.ntheta;
-    double cx[8], cy[8];
-    cart_dirs(cx, cy);
-    for (long long s = (long long)A.m0 * A.nr + blockIdx.x * (long long)blockDim.x + threadIdx.x;
-         s < (long long)A.m1 * A.nr; s += (long long)gridDim.x * blockDim.x) {
-        const int m = (int)(s / A.nr), j = (int)(s - (long long)m * A.nr);
-        const real *fp = A.f + (long long)m * A.ld + j;
-        double fv[NV];
-        for (int q = 0; q < NV; ++q) fv[q] = (double)fp[(long long)q * A.plane];
-        double rho = fv[0], jx = 0.0, jy = 0.0;
-        for (int k = 0; k < 4; ++k)
-            for (int i = 0; i < 8; ++i) {
-                rho += fv[1 + 8 * k + i];
-                jx += fv[1 + 8 * k + i] * A.v[k] * cx[i];
-                jy += fv[1 + 8 * k + i] * A.v[k] * cy[i];
-            }
-        const double ux = jx / rho, uy = jy / rho;
-        double sth, cth;
-        sincospi(A.th_over_pi * m, &sth, &cth);
-        double M[12] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
-        for (int q = 0; q < NV; ++q) {
-            const int k = q == 0 ? -1 : (q - 1) / 8, i = q == 0 ? 0 : (q - 1) % 8;
-            const double vx = k < 0 ? 0.0 : A.v[k] * cx[i], vy = k < 0 ? 0.0 : A.v[k] * cy[i];
-            const double dx = vx - ux, dy = vy - uy;
-            const double a = dx * cth + dy * sth, b = -dx * sth + dy * cth;  // v* polar
-            const double g = fv[q], s2 = a * a + b * b;
-            M[0] += g * a * a;
-            M[1] += g * a * b;
-            M[2] += g * b * b;
-            M[3] += g * a * a * a;
-            M[4] += g * a * a * b;
-            M[5] += g * a * b * b;
-            M[6] += g * b * b * b;
-            M[7] += 0.5 * g * s2 * a;
-            M[8] += 0.5 * g * s2 * b;
-            M[9] += 0.5 * g * s2 * a * a;
-            M[10] += 0.5 * g * s2 * a * b;
-            M[11] += 0.5 * g * s2 * b * b;
+    const long long first = (long long)A.m0 * A.nr, end = (long long)A.m1 * A.nr;
+    for (long long base = first + blockIdx.x * 256LL; base < end; base += gridDim.x * 256LL) {
+        const int row0 = (int)(base / A.nr);
+        const int rows = (int)((min(base + 256, end) - 1) / A.nr) - row0 + 1;
+        for (int t = threadIdx.x; t < 3 * rows; t += 256) {
+            const int r = t / 3, n = t - 3 * r;
+            sincospi((n + 1) * (A.th_over_pi * (row0 + r)), &trig[r][2 * n + 1], &trig[r][2 * n]);
         }
-        const double T = 0.5 * (M[0] + M[2]) / rho;  // f's own temperature
-        M[0] -= rho * T;
-        M[2] -= rho * T;
-        M[9] -= 2.0 * rho * T * T;
-        M[11] -= 2.0 * rho * T * T;
-        for (int c = 0; c < 12; ++c) A.out[c * N + s] = M[c];
+        __syncthreads();
+        const long long s = base + threadIdx.x;
+        if (s < end) {
+            const int m = (int)(s / A.nr), j = (int)(s - (long long)m * A.nr);
+            const real *fp = A.f + (long long)m * A.ld + j;
+            real fv[NV];
+#pragma unroll
+            for (int q = 0; q < NV; ++q) fv[q] = fp[(long long)q * A.plane];
+            // sums over the rings: order 0, 1, 2 (trace and second harmonic), 3
+            // (first and third harmonic), 4 (trace and second harmonic)
+            double rho = widen(fv[0]), jx = 0.0, jy = 0.0, E2 = 0.0, X2 = 0.0, Y2 = 0.0;
+            double A1 = 0.0, B1 = 0.0, A3 = 0.0, B3 = 0.0, E4 = 0.0, X4 = 0.0, Y4 = 0.0;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                double g[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) g[i] = widen(fv[1 + 8 * k + i]);
+                const RingHarmonics h = ring_harmonics(g);
+                rho += h.s0;
+                jx = fma(A.v[k], h.c1, jx);
+                jy = fma(A.v[k], h.s1, jy);
+                E2 = fma(A.v2[k], h.s0, E2);
+                X2 = fma(A.v2[k], h.c2, X2);
+                Y2 = fma(A.v2[k], h.s2, Y2);
+                A1 = fma(A.v3[k], h.c1, A1);
+                B1 = fma(A.v3[k], h.s1, B1);
+                A3 = fma(A.v3[k], h.c3, A3);
+                B3 = fma(A.v3[k], h.s3, B3);
+                E4 = fma(A.v4[k], h.s0, E4);
+                X4 = fma(A.v4[k], h.c2, X4);
+                Y4 = fma(A.v4[k], h.s2, Y4);
+            }
+            // into the polar frame
+            const double *t = trig[m - row0];
+            auto turn = [](double &x, double &y, double c, double sn) {
+                const double a = fma(x, c, y * sn);
+                y = fma(y, c, -(x * sn));
+                x = a;
+            };
+            turn(jx, jy, t[0], t[1]);
+            turn(A1, B1, t[0], t[1]);
+            turn(X2, Y2, t[2], t[3]);
+            turn(X4, Y4, t[2], t[3]);
+            turn(A3, B3, t[4], t[5]);
+            const double inv_rho = 1.0 / rho;
+            const double U = jx * inv_rho, V = jy * inv_rho;
+            const double UU = U * U, UV = U * V, VV = V * V, u2 = UU + VV;
+            // M*_2 (central): rr, r-theta, theta-theta
+            const double rr = fma(-rho, UU, 0.5 * (E2 + X2)), rt = fma(-rho, UV, 0.5 * Y2),
+                         tt = fma(-rho, VV, 0.5 * (E2 - X2));
+            // M*_3: raw third moment less u's products with M*_2 and rho u u u
+            const double c3 = fma(rho, UU, 3.0 * rr), d3 = fma(rho, VV, 3.0 * tt);
+            const double rrr = fma(-U, c3, 0.25 * fma(3.0, A1, A3));
+            const double ttt = fma(-V, d3, 0.25 * fma(3.0, B1, -B3));
+            const double rrt = fma(-V, fma(rho, UU, rr), fma(-2.0 * U, rt, 0.25 * (B1 + B3)));
+            const double rtt = fma(-U, fma(rho, VV, tt), fma(-2.0 * V, rt, 0.25 * (A1 - A3)));
+            const double q_r = rrr + rtt, q_t = rrt + ttt;  // sum f |v*|^2 v*
+            // 2 M*_{4,2}: sum f |v|^2 v v less what u contributes
+            const double tr = rr + tt, w_r = fma(U, rr, V * rt), w_t = fma(U, rt, V * tt);
+            const double z = fma(rho, u2, tr);
+            const double h_r = q_r + 2.0 * w_r, h_t = q_t + 2.0 * w_t;
+            const double f_rr = fma(-UU, z, 0.5 * (E4 + X4)) - 2.0 * fma(U, h_r, fma(U, rrr, V * rrt)) - u2 * rr;
+            const double f_tt = fma(-VV, z, 0.5 * (E4 - X4)) - 2.0 * fma(V, h_t, fma(U, rtt, V * ttt)) - u2 * tt;
+            const double f_rt = fma(-UV, z, 0.5 * Y4) - fma(V, h_r, U * h_t) - 2.0 * fma(U, rrt, V * rtt) - u2 * rt;
+            // less the Maxwellian's: rho T = half the trace, 2 rho T^2
+            const double rT = 0.5 * tr, rTT2 = 2.0 * rT * (rT * inv_rho);
+            double *out = A.out + s;
+            out[0] = rr - rT;
+            out[N] = rt;
+            out[2 * N] = tt - rT;
+            out[3 * N] = rrr;
+            out[4 * N] = rrt;
+            out[5 * N] = rtt;
+            out[6 * N] = ttt;
+            out[7 * N] = 0.5 * q_r;
+            out[8 * N] = 0.5 * q_t;
+            out[9 * N] = fma(0.5, f_rr, -rTT2);
+            out[10 * N] = 0.5 * f_rt;
+            out[11 * N] = fma(0.5, f_tt, -rTT2);
+        }
+        __syncthreads();
     }
 }
 

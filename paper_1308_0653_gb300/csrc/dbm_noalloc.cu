@@ -65,8 +65,8 @@ unsigned long long current_context_id()
 const double kPi = 3.14159265358979323846;
 
 // One CTA per theta row: each site's sums rho, jx, jy, e2 = sum f |v|^2 from
-// its 33 f (Sec. II.B, Cartesian components) -- in FP32 ring by ring as the
-// step and dbm_moments compute them, or in FP64 -- weighted by r and summed
+// its 33 f (Sec. II.B, Cartesian components), ring by ring in the state's
+// precision as the step and dbm_moments compute them, weighted by r and summed
 // in FP64 into the row's 4 partials {mass, px, py, energy}, times dr dtheta
 // (energy rho T + rho u^2 / 2 = e2 / 2 for D = 2).  f: [33][ntheta][ld].
 template <typename real>
@@ -83,22 +83,7 @@ __global__ void __launch_bounds__(256) row_totals_kernel(const real *f, int nr, 
 #pragma unroll
         for (int q = 0; q < dbm::NV; ++q) fv[q] = fp[(long long)q * plane];
         real rho, jx, jy, e2;
-        if constexpr (sizeof(real) == 4) {
-            dbm::ring_moments<real>(fv, vv.v, vv.v2, rho, jx, jy, e2);
-        } else {
-            double cx[8], cy[8];
-            dbm::cart_dirs(cx, cy);
-            rho = fv[0];
-            jx = jy = e2 = 0.0;
-            for (int k = 0; k < 4; ++k)
-                for (int i = 0; i < 8; ++i) {
-                    const double fq = fv[1 + 8 * k + i];
-                    rho += fq;
-                    jx += fq * vv.v[k] * cx[i];
-                    jy += fq * vv.v[k] * cy[i];
-                    e2 += fq * vv.v2[k];
-                }
-        }
+        dbm::ring_moments<real>(fv, vv.v, vv.v2, rho, jx, jy, e2);
         const double r = r_in + (j + 0.5) * dr;
         acc[0] += (double)rho * r;
         acc[1] += (double)jx * r;
