@@ -115,6 +115,20 @@ void weight_coeffs(const double v[4], double Fc[4][4])
     }
 }
 
+RingPowers<double> ring_powers(const double v[4])
+{
+    RingPowers<double> x;
+    for (int k = 0; k < 4; ++k) {
+        const double v3 = v[k] * v[k] * v[k], v4 = v3 * v[k];
+        x.v3_6[k] = v3 / 6.0;
+        x.v3_2[k] = v3 / 2.0;
+        x.v4_24[k] = v4 / 24.0;
+        x.v4_6[k] = v4 / 6.0;
+        x.v5_24[k] = v4 * v[k] / 24.0;
+    }
+    return x;
+}
+
 // cos and sin of (i pi/4 - theta_m); with ntheta a multiple of 8 the angle is
 // taken from the integer index (i ntheta/8 - m) mod ntheta, so the table is
 // exactly invariant under the pi/4 rotation (m -> m + ntheta/8, i -> i + 1).
@@ -165,6 +179,8 @@ struct dbm_s {
     int grid, rows_per_item, items;
     StepArgs<float> a32[2];   // [0]: f0 -> f1, [1]: f1 -> f0
     StepArgs<double> a64[2];
+    Direct64Args d64[2];      // FP64 variant 2: the direct kernel's arguments
+    bool direct;
     cudaGraphExec_t graph;    // GRAPH_STEPS steps starting from buffer 0
     int device;
     bool tmap_ok;             // tensor maps encoded (tensor-TMA variants usable)
@@ -292,6 +308,7 @@ void fill_step_args(dbm_t *h, StepArgs<real> (&a)[2])
         A.c.m_exp = (real)p.m;
         A.c.n_exp = (real)p.n;
         A.c.T_th = (real)p.T_th;
+        if constexpr (std::is_same<real, double>::value) static_cast<RingPowers<real> &>(A.c) = ring_powers(p.v);
         for (int k = 0; k < 4; ++k) {
             A.c.v[k] = (real)p.v[k];
             A.c.v2[k] = (real)(p.v[k] * p.v[k]);
@@ -334,8 +351,9 @@ int upload_tables(dbm_t *h)
 
 int launch_one(dbm_t *h, int b, cudaStream_t s)
 {
-    cudaError_t e = h->p.precision == DBM_FP64 ? launch_step<double>(h->variant, h->a64[b], h->grid, s)
-                                               : launch_step<float>(h->variant, h->a32[b], h->grid, s);
+    cudaError_t e = h->direct ? launch_direct64(h->d64[b], s)
+                    : h->p.precision == DBM_FP64 ? launch_step<double>(h->variant, h->a64[b], h->grid, s)
+                                                 : launch_step<float>(h->variant, h->a32[b], h->grid, s);
     if (e != cudaSuccess) return cuda_fail(e, "step kernel launch");
     return DBM_OK;
 }
@@ -387,6 +405,27 @@ int pick_variant(const dbm_params &p)
     return p.precision == DBM_FP64 ? default_variant<double>() : default_variant<float>();
 }
 
+// The direct kernel's tasks: FP64 variant 2 of a single simulation (a batch runs
+// the row ring for it).  A warp task is 32 sites of a row; the SM quarters
+// (4 per SM) each take one at a time.  Whole waves of quarters run full tasks; of
+// the rest, quarter tasks (0.42 of a full one's time each, 4 per task) where
+// they finish first: up to two waves of them against one of full tasks.
+void fill_direct64(dbm_t *h, int nsm)
+{
+    const dbm_params &p = h->p;
+    const long long chunks = (p.nr + 31) / 32, tasks = chunks * p.ntheta, quarters = 4LL * nsm;
+    h->direct = p.precision == DBM_FP64 && h->variant == default_variant<double>() && tasks <= (1 << 29);
+    if (!h->direct) return;
+    long long full = tasks / quarters * quarters;
+    if (4 * (tasks - full) > 2 * quarters) full = tasks;
+    for (int b = 0; b < 2; ++b) {
+        h->d64[b].A = h->a64[b];
+        h->d64[b].chunks = (int)chunks;
+        h->d64[b].full = (int)full;
+        h->d64[b].quarters = (int)quarters;
+    }
+}
+
 // Launch shape for a kernel variant: persistent CTAs, one per resident slot,
 // and the rows per item above unless the parameters fix them.
 int configure_launch(dbm_t *h, int variant)
@@ -433,6 +472,7 @@ int configure_launch(dbm_t *h, int variant)
         fill_step_args<double>(h, h->a64);
     else
         fill_step_args<float>(h, h->a32);
+    fill_direct64(h, nsm);
     if (h->graph) {
         cudaGraphExecDestroy(h->graph);
         h->graph = nullptr;
@@ -698,8 +738,10 @@ static cudaError_t launch_init_as(dbm_t *h, const double *d_fields, cudaStream_t
     A.m1 = m1;
     for (int k = 0; k < 4; ++k) {
         A.v[k] = (real)h->p.v[k];
+        A.v2[k] = (real)(h->p.v[k] * h->p.v[k]);
         for (int c = 0; c < 4; ++c) A.Fc[k][c] = (real)Fc[k][c];
     }
+    if constexpr (std::is_same<real, double>::value) static_cast<RingPowers<real> &>(A) = ring_powers(h->p.v);
     return launch_init<real>(A, s);
 }
 

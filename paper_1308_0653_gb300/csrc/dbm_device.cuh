@@ -56,12 +56,18 @@ template <typename real> struct Halo;
 template <> struct Halo<float> { static constexpr int value = 4; };   // 16 bytes
 template <> struct Halo<double> { static constexpr int value = 2; };  // 16 bytes
 
+// Powers of the ring speeds for the FP64 update; nothing for FP32.
+template <typename real> struct RingPowers {};
+template <> struct RingPowers<double> {
+    double v3_6[4], v3_2[4], v4_24[4], v4_6[4], v5_24[4];  // v^3/6, v^3/2, v^4/24, v^4/6, v^5/24
+};
+
 // Per-instance constants of the update (host-computed in double, rounded to
 // real).  A single-instance launch reads them from its parameter block (the
 // constant bank, as instruction operands); a batched launch reads them from
 // a constant-memory table indexed by the item's slot.
 template <typename real>
-struct StepConsts {
+struct StepConsts : RingPowers<real> {
     real cr_scale;        // dt / dr
     real ct_scale;        // dt / dtheta
     real decay;           // exp(-dt / tau)
@@ -496,25 +502,17 @@ __device__ __forceinline__ void site_update(const StepArgs<real> &A, const StepC
     //     with f^eq (1 - E + dt M / f^eq) = poly(xi) (beta_k - gamma_k xi) in ring k
     real *out = A.f_out + (long long)m * A.ld + j;
     out[0] = O::fma(A0, beta0, O::mul(C.decay, REREAD ? sc[col] : f[0]));
-    if constexpr (sizeof(real) == 8 || !DIR_OUTER) {
+    if constexpr (!DIR_OUTER) {
         // Ring by ring with the geometry of all 8 directions held: the
-        // single-instance kernels and FP64.
+        // single-instance kernels.
         real ar[8], at[8], sa[8];
         int rn[8], tn[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             // as geom(i, ...), written out: the compiler schedules this form better
-            if (sizeof(real) == 8 && i >= 4) {
-                // FP64: the trig table holds direction i + 4 as the exact
-                // negation of direction i, so the magnitudes are the same bits
-                ar[i] = ar[i - 4];
-                at[i] = at[i - 4];
-                sa[i] = sa[i - 4];
-            } else {
-                ar[i] = O::mul(fabs(cs[i]), C.cr_scale);
-                at[i] = O::mul(O::mul(fabs(sn8[i]), C.ct_scale), inv_r);
-                sa[i] = O::add(ar[i], at[i]);
-            }
+            ar[i] = O::mul(fabs(cs[i]), C.cr_scale);
+            at[i] = O::mul(O::mul(fabs(sn8[i]), C.ct_scale), inv_r);
+            sa[i] = O::add(ar[i], at[i]);
             int o = cs[i] >= real(0) ? -1 : 1;  // C_r >= 0: backward difference
             if (j == 0 && o < 0) {
                 o = C.centre == 1 ? (((i + 4) & 7) - i) * WP : (C.centre == 2 ? -1 : 0);
@@ -555,41 +553,14 @@ __device__ __forceinline__ void site_update(const StepArgs<real> &A, const StepC
                 t = O::fma(vk, adv, t);
                 out[(long long)q * A.plane] = t;
             };
-            if constexpr (sizeof(real) == 8) {
-                // FP64 is bound by its arithmetic: opposite directions i and
-                // i+4 have xi and -xi, so the polynomial splits into an even
-                // part E and an odd part O evaluated once, poly(+-xi) = E +- O;
-                // they also share |C_r| + |C_theta|, so the weight of the
-                // site's own f, E - v_k (|C_r| + |C_theta|), is taken once
-                auto update_pair_one = [&](int i, real xi, real poly, real keep) {
-                    const int q = 1 + 8 * k + i;
-                    real t = O::mul(poly, O::fma(-gamma, xi, beta));
-                    const real fq = REREAD ? sc[q * WP + col] : f[q];
-                    t = O::fma(keep, fq, t);
-                    const real adv = O::fma(ar[i], sc[q * WP + rn[i]], O::mul(at[i], sc[q * WP + tn[i]]));
-                    t = O::fma(vk, adv, t);
-                    out[(long long)q * A.plane] = t;
-                };
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const real xi = O::mul(vk, w[i]);
-                    const real x2 = O::mul(xi, xi);
-                    const real Ev = O::fma(x2, O::fma(x2, real(1.0 / 24.0), A2), A0);
-                    const real Od = O::mul(xi, O::fma(x2, real(1.0 / 6.0), A1));
-                    const real keep = O::fma(-vk, sa[i], C.decay);
-                    update_pair_one(i, xi, O::add(Ev, Od), keep);
-                    update_pair_one(i + 4, -xi, O::sub(Ev, Od), keep);
-                }
-            } else {
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const real xi = O::mul(vk, w[i]);
-                    update_one(i, xi, O::fma(xi, O::fma(xi, O::fma(xi, O::fma(xi, real(1.0 / 24.0), real(1.0 / 6.0)), A2), A1), A0));
-                }
+            for (int i = 0; i < 8; ++i) {
+                const real xi = O::mul(vk, w[i]);
+                update_one(i, xi, O::fma(xi, O::fma(xi, O::fma(xi, O::fma(xi, real(1.0 / 24.0), real(1.0 / 6.0)), A2), A1), A0));
             }
         }
     } else {
-        // FP32 with DIR_OUTER (batched launches, which hold each instance's
+        // DIR_OUTER (batched launches, which hold each instance's
         // constants in registers): direction by direction, so that only one
         // direction's geometry is live at a time.  Each velocity's arithmetic
         // is the ring-by-ring one, operation for operation: same bits.
@@ -635,26 +606,25 @@ __device__ __forceinline__ void site_update(const StepArgs<real> &A, const StepC
     const real lt = (uth >= real(0) ? sp : sn)[LAMOFF + col];
     const real tr = O::mul(O::mul(fabs(ur), C.cr_scale), O::sub(lst, lr));
     const real tt = O::mul(O::mul(O::mul(fabs(uth), C.ct_scale), inv_r), O::sub(lst, lt));
-    real ln;
-    if constexpr (sizeof(real) == 4) {
-        // y - dlam - tr - tt summed exactly, then rounded without bias
-        float sum, err, e2;
-        two_sum_f(lst, -dlam, sum, err);
-        two_sum_f(sum, -tr, sum, e2);
-        err = __fadd_rn(err, e2);
-        two_sum_f(sum, -tt, sum, e2);
-        err = __fadd_rn(err, e2);
-        const uint32_t site = (uint32_t)m * (uint32_t)A.ld + (uint32_t)j;
-        const float u = (float)(hash32(site * 0x9e3779b9u ^ __float_as_uint(lst)) >> 8) * 0x1p-24f;
-        ln = round_stochastic_unit(sum, err, u);
-    } else {
-        ln = kY ? O::sub(lst, dlam) : O::add(lst, dlam);
-        ln = O::sub(ln, tr);
-        ln = O::sub(ln, tt);
-    }
+    // y - dlam - tr - tt summed exactly, then rounded without bias
+    float sum, err, e;
+    two_sum_f(lst, -dlam, sum, err);
+    two_sum_f(sum, -tr, sum, e);
+    err = __fadd_rn(err, e);
+    two_sum_f(sum, -tt, sum, e);
+    err = __fadd_rn(err, e);
+    const uint32_t site = (uint32_t)m * (uint32_t)A.ld + (uint32_t)j;
+    const float u = (float)(hash32(site * 0x9e3779b9u ^ __float_as_uint(lst)) >> 8) * 0x1p-24f;
+    real ln = round_stochastic_unit(sum, err, u);
     ln = fmin(fmax(ln, real(0)), real(1));
     A.lam_out[(long long)m * A.ld + j] = ln;
 }
+
+}  // namespace dbm
+
+#include "dbm_update64.cuh"
+
+namespace dbm {
 
 // ---------------------------------------------------------------------------
 // Full disc (centre == 2, Sec. II.D with a full 2 pi grid): the inner ghost of
@@ -860,7 +830,17 @@ __device__ __forceinline__ void march(const Work &work, unsigned char *smem_raw,
                 }
             }
             const int m = mb + c - 1;
-            if (active && !abort_flag) {
+            if constexpr (sizeof(real) == 8) {  // every lane takes part (idle ones store nothing)
+                if (!abort_flag) {
+                    const bool ghost = C.centre == 2 && j == 0;
+                    if (ghost) fill_centre_ghost<real, WP, NV * WP, HALO>(A, sm + (P % NSTAGE) * SLOT, m);
+                    __syncwarp();
+                    site_update64_ring<WP, NV * WP, HALO>(A, C, sm + ((P - 1) % NSTAGE) * SLOT,
+                                                          sm + (P % NSTAGE) * SLOT, sm + ((P + 1) % NSTAGE) * SLOT,
+                                                          j0, tx, m, A.rowtab + (long long)m * 16);
+                    if (ghost) fence_proxy_async_smem();
+                }
+            } else if (active && !abort_flag) {
                 real cs[8], sn8[8];
                 const real *rt = A.rowtab + (long long)m * 16;
 #pragma unroll
@@ -1106,7 +1086,16 @@ __device__ __forceinline__ void march2(const Work &work, unsigned char *smem_raw
                     return;
                 }
                 const real *sc = sm + (P % NSTAGE) * SLOT;
-                if (active) {
+                if constexpr (sizeof(real) == 8) {  // every lane takes part (idle ones store nothing)
+                    const bool ghost = C.centre == 2 && j == 0;
+                    if (ghost)
+                        fill_centre_ghost<real, WP, LAMOFF, HALO>(A, sm + (P % NSTAGE) * SLOT, mb + c - 1);
+                    __syncwarp();
+                    site_update64_ring<WP, LAMOFF, HALO>(A, C, sm + ((P - 1) % NSTAGE) * SLOT, sc,
+                                                         sm + ((P + 1) % NSTAGE) * SLOT, j0, tx, mb + c - 1,
+                                                         sc + RTOFF);
+                    if (ghost) fence_proxy_async_smem();
+                } else if (active) {
                     real cs[8], sn8[8];
                     const real *rt = sc + RTOFF;
 #pragma unroll
@@ -1238,7 +1227,7 @@ static __global__ void rcp_selftest_kernel(const float *x, float *approx, float 
 // as DBM_EINVAL (the state is then undefined).
 // ---------------------------------------------------------------------------
 template <typename real>
-struct InitArgs {
+struct InitArgs : RingPowers<real> {
     const double *fields;
     real *f;
     real *lam;
@@ -1247,7 +1236,7 @@ struct InitArgs {
     long long plane;
     int nr, ntheta, ld;
     int m0, m1;          // theta rows [m0, m1) of this launch
-    real v[4];
+    real v[4], v2[4];
     real Fc[4][4];
 };
 
@@ -1290,17 +1279,34 @@ __global__ void __launch_bounds__(256) init_kernel(const InitArgs<real> A)
         const real w[4] = {wx, O::mul(H, O::add(wx, wy)), wy, O::mul(H, O::sub(wy, wx))};
         real *out = A.f + (long long)m * A.ld + j;
         out[0] = O::mul(O::mul(rho, F0), A0);
+        if constexpr (sizeof(real) == 8) {
+            // bound by FP64 instructions: E(w^2) +- w O(w^2) as in site_update64
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const real rF = O::mul(rho, F[k]);
+            for (int k = 0; k < 4; ++k) {
+                const double rF = rho * F[k];
+                const double e0 = rF * A0, o0 = A.v[k] * (rF * A1), e1 = A.v2[k] * (rF * A2);
+                const double o1 = rF * A.v3_6[k], e4 = rF * A.v4_24[k];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const real xi = O::mul(A.v[k], w[i]);  // direction i + 4 has -xi
-                const real x2 = O::mul(xi, xi);
-                const real Ev = O::fma(x2, O::fma(x2, real(1.0 / 24.0), A2), A0);
-                const real Od = O::mul(xi, O::fma(x2, real(1.0 / 6.0), A1));
-                out[(long long)(1 + 8 * k + i) * A.plane] = O::mul(rF, O::add(Ev, Od));
-                out[(long long)(5 + 8 * k + i) * A.plane] = O::mul(rF, O::sub(Ev, Od));
+                for (int i = 0; i < 4; ++i) {
+                    const double w2 = w[i] * w[i];
+                    const double Ev = fma(w2, fma(w2, e4, e1), e0), Od = fma(w2, o1, o0);
+                    out[(long long)(1 + 8 * k + i) * A.plane] = fma(w[i], Od, Ev);
+                    out[(long long)(5 + 8 * k + i) * A.plane] = fma(-w[i], Od, Ev);
+                }
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const real rF = O::mul(rho, F[k]);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const real xi = O::mul(A.v[k], w[i]);  // direction i + 4 has -xi
+                    const real x2 = O::mul(xi, xi);
+                    const real Ev = O::fma(x2, O::fma(x2, real(1.0 / 24.0), A2), A0);
+                    const real Od = O::mul(xi, O::fma(x2, real(1.0 / 6.0), A1));
+                    out[(long long)(1 + 8 * k + i) * A.plane] = O::mul(rF, O::add(Ev, Od));
+                    out[(long long)(5 + 8 * k + i) * A.plane] = O::mul(rF, O::sub(Ev, Od));
+                }
             }
         }
         A.lam[(long long)m * A.ld + j] = (real)LamStore<real>::from_lambda(lam_d);

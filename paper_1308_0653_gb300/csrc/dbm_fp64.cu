@@ -1,9 +1,9 @@
 // FP64 kernels (ALU-bound on GB300).  Variants as in the FP32 unit:
 //   1  v1  64  5  no   2
-//   2  v2  64  5  no   2
-//   3  v2  64  4  yes  3
+//   2  v2  64  5  no   2   (a single simulation runs the direct kernel instead)
+//   3  v2  64  4       3
 //   4  v3  64  5  no   2   (tensor-map TMA)
-//   5  v3  64  4  yes  3   (tensor-map TMA)
+//   5  v3  64  4       3   (tensor-map TMA)
 #include "dbm.h"
 #define DBM_REAL double
 #define DBM_VARIANTS(X) X(1, 1, 64, 5, false, 2) X(2, 2, 64, 5, false, 2) X(3, 2, 64, 4, true, 3) \
@@ -12,3 +12,18 @@
 #define DBM_FALLBACK_VARIANT 2
 #define DBM_BATCH_CONST_SLOTS DBM_BATCH_CONST_FP64  // batch constant table entries (304 B each)
 #include "dbm_launch_impl.cuh"
+
+namespace dbm {
+cudaError_t launch_direct64(const Direct64Args &D, cudaStream_t s)
+{
+    // up to two waves of warps, each has an SM quarter (nearly) to itself and
+    // its loads are not hidden by others
+    const long long tasks = (long long)D.chunks * D.A.ntheta;
+    const unsigned blocks = (unsigned)((D.full + 3) / 4 + tasks - D.full);
+    if (tasks <= 2 * D.quarters)
+        direct64_kernel<true><<<blocks, 128, 0, s>>>(D);
+    else
+        direct64_kernel<false><<<blocks, 128, 0, s>>>(D);
+    return cudaGetLastError();
+}
+}  // namespace dbm
