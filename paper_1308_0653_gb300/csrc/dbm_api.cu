@@ -165,6 +165,14 @@ void row_angles(const dbm_params &p, int m, double c[8], double s[8])
 
 }  // namespace
 
+// How a single simulation steps.  The default variant of a precision runs the
+// row ring where that is the fastest, other kernels (the same update, bit for
+// bit) elsewhere; every other variant always runs its own kernel.
+enum Path {
+    PATH_RING,      // the variant's row-ring kernel
+    PATH_DIRECT64,  // FP64: straight from global memory
+};
+
 struct dbm_s {
     dbm_params p;
     Layout L;
@@ -179,8 +187,9 @@ struct dbm_s {
     int grid, rows_per_item, items;
     StepArgs<float> a32[2];   // [0]: f0 -> f1, [1]: f1 -> f0
     StepArgs<double> a64[2];
-    Direct64Args d64[2];      // FP64 variant 2: the direct kernel's arguments
-    bool direct;
+    Direct64Args d64[2];      // the FP64 direct kernel's arguments
+    Path path;                // how the chosen variant steps this simulation
+    int nsm;
     cudaGraphExec_t graph;    // GRAPH_STEPS steps starting from buffer 0
     int device;
     bool tmap_ok;             // tensor maps encoded (tensor-TMA variants usable)
@@ -192,7 +201,7 @@ struct dbm_s {
 
 namespace {
 
-constexpr int GRAPH_STEPS = 32;
+constexpr int GRAPH_STEPS = 32;  // an even number of passes on every path (see Path)
 
 // Second word of the status region: set by the init kernel when an initial
 // field value is invalid (rho <= 0, T <= 0, not finite).
@@ -251,6 +260,12 @@ bool encode_maps(const dbm_t *h, StepArgs<real> &A)
     const cuuint32_t one3[3] = {1, 1, 1};
     if (enc(&A.tm_f, dt, 3, (void *)A.f_in, gdim3, gstr3, box3, one3, CU_TENSOR_MAP_INTERLEAVE_NONE,
             CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return false;
+    const cuuint32_t box_out[3] = {32, 1, (cuuint32_t)NV};
+    if (sizeof(real) == 4 &&
+        enc(&A.tm_out, dt, 3, (void *)A.f_out, gdim3, gstr3, box_out, one3, CU_TENSOR_MAP_INTERLEAVE_NONE,
+            CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return false;
     const cuuint64_t gdim2[2] = {(cuuint64_t)h->p.nr, (cuuint64_t)h->p.ntheta};
@@ -349,12 +364,32 @@ int upload_tables(dbm_t *h)
     return DBM_OK;
 }
 
-int launch_one(dbm_t *h, int b, cudaStream_t s)
+// One pass over the state from buffer b to the other: *took of the `left` steps.
+int launch_pass(dbm_t *h, int b, int64_t left, cudaStream_t s, int *took)
 {
-    cudaError_t e = h->direct ? launch_direct64(h->d64[b], s)
-                    : h->p.precision == DBM_FP64 ? launch_step<double>(h->variant, h->a64[b], h->grid, s)
-                                                 : launch_step<float>(h->variant, h->a32[b], h->grid, s);
+    cudaError_t e;
+    *took = 1;
+    switch (h->path) {
+    case PATH_DIRECT64: e = launch_direct64(h->d64[b], s); break;
+    default:
+        e = h->p.precision == DBM_FP64 ? launch_step<double>(h->variant, h->a64[b], h->grid, s)
+                                       : launch_step<float>(h->variant, h->a32[b], h->grid, s);
+    }
     if (e != cudaSuccess) return cuda_fail(e, "step kernel launch");
+    return DBM_OK;
+}
+
+// nsteps steps, pass by pass.
+int run_passes(dbm_t *h, int64_t nsteps, cudaStream_t s)
+{
+    while (nsteps > 0) {
+        int took = 0;
+        const int rc = launch_pass(h, h->cur, nsteps, s, &took);
+        if (rc != DBM_OK) return rc;
+        h->cur ^= 1;
+        nsteps -= took;
+        h->steps += took;
+    }
     return DBM_OK;
 }
 
@@ -366,7 +401,9 @@ int build_graph(dbm_t *h)
     cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
     int rc = DBM_OK;
     if (e == cudaSuccess) {
-        for (int s = 0; s < GRAPH_STEPS && rc == DBM_OK; ++s) rc = launch_one(h, s & 1, cs);
+        int took = 0;
+        for (int s = 0, b = 0; s < GRAPH_STEPS && rc == DBM_OK; s += took, b ^= 1)
+            rc = launch_pass(h, b, GRAPH_STEPS - s, cs, &took);
         e = cudaStreamEndCapture(cs, &g);
     }
     if (e == cudaSuccess && rc == DBM_OK) e = cudaGraphInstantiate(&h->graph, g, 0);
@@ -405,17 +442,14 @@ int pick_variant(const dbm_params &p)
     return p.precision == DBM_FP64 ? default_variant<double>() : default_variant<float>();
 }
 
-// The direct kernel's tasks: FP64 variant 2 of a single simulation (a batch runs
-// the row ring for it).  A warp task is 32 sites of a row; the SM quarters
-// (4 per SM) each take one at a time.  Whole waves of quarters run full tasks; of
-// the rest, quarter tasks (0.42 of a full one's time each, 4 per task) where
-// they finish first: up to two waves of them against one of full tasks.
-void fill_direct64(dbm_t *h, int nsm)
+// The FP64 direct kernel's tasks.  A warp task is 32 sites of a row; the SM
+// quarters (4 per SM) each take one at a time.  Whole waves of quarters run full
+// tasks; of the rest, quarter tasks (0.42 of a full one's time each, 4 per task)
+// where they finish first: up to two waves of them against one of full tasks.
+void fill_direct64(dbm_t *h)
 {
     const dbm_params &p = h->p;
-    const long long chunks = (p.nr + 31) / 32, tasks = chunks * p.ntheta, quarters = 4LL * nsm;
-    h->direct = p.precision == DBM_FP64 && h->variant == default_variant<double>() && tasks <= (1 << 29);
-    if (!h->direct) return;
+    const long long chunks = (p.nr + 31) / 32, tasks = chunks * p.ntheta, quarters = 4LL * h->nsm;
     long long full = tasks / quarters * quarters;
     if (4 * (tasks - full) > 2 * quarters) full = tasks;
     for (int b = 0; b < 2; ++b) {
@@ -424,6 +458,17 @@ void fill_direct64(dbm_t *h, int nsm)
         h->d64[b].full = (int)full;
         h->d64[b].quarters = (int)quarters;
     }
+}
+
+// The path of the handle's variant.
+Path pick_path(const dbm_t *h)
+{
+    const dbm_params &p = h->p;
+    const long long warps = (long long)((p.nr + 31) / 32) * p.ntheta;
+    if (p.precision == DBM_FP64)
+        return h->variant == default_variant<double>() && warps <= (1 << 29) ? PATH_DIRECT64 : PATH_RING;
+    if (h->variant != default_variant<float>()) return PATH_RING;
+    return PATH_RING;
 }
 
 // Launch shape for a kernel variant: persistent CTAs, one per resident slot,
@@ -472,7 +517,9 @@ int configure_launch(dbm_t *h, int variant)
         fill_step_args<double>(h, h->a64);
     else
         fill_step_args<float>(h, h->a32);
-    fill_direct64(h, nsm);
+    h->nsm = nsm;
+    h->path = pick_path(h);
+    if (h->path == PATH_DIRECT64) fill_direct64(h);
     if (h->graph) {
         cudaGraphExecDestroy(h->graph);
         h->graph = nullptr;
@@ -846,11 +893,12 @@ int dbm_step(dbm_t *h, int64_t nsteps, void *stream)
             nsteps -= GRAPH_STEPS;
             h->steps += GRAPH_STEPS;
         } else {
-            int rc = launch_one(h, h->cur, s);
+            int took = 0;
+            int rc = launch_pass(h, h->cur, nsteps, s, &took);
             if (rc != DBM_OK) return rc;
             h->cur ^= 1;
-            nsteps -= 1;
-            h->steps += 1;
+            nsteps -= took;
+            h->steps += took;
         }
     }
     note_work(h, s);
@@ -1152,18 +1200,10 @@ int dbm_autotune(dbm_t *h, int steps, void *stream, int *best, float *ms_per_ste
             continue;
         }
         // two untimed steps, then `steps` timed single launches
-        for (int k = 0; k < 2 && rc == DBM_OK; ++k) {
-            rc = launch_one(h, h->cur, s);
-            h->cur ^= 1;
-            h->steps += 1;
-        }
+        rc = run_passes(h, 2, s);
         if (rc != DBM_OK) break;
         cudaEventRecord(e0, s);
-        for (int k = 0; k < steps && rc == DBM_OK; ++k) {
-            rc = launch_one(h, h->cur, s);
-            h->cur ^= 1;
-            h->steps += 1;
-        }
+        rc = run_passes(h, steps, s);
         cudaEventRecord(e1, s);
         cudaError_t e = cudaEventSynchronize(e1);
         if (e != cudaSuccess) {

@@ -91,6 +91,7 @@ template <typename real>
 struct StepArgs {
     CUtensorMap tm_f;     // 128 B, 64-byte aligned
     CUtensorMap tm_lam;
+    CUtensorMap tm_out;   // this parity's output f, box of one row of 32 columns (FP32)
     const real *f_in;
     real *f_out;
     const real *lam_in;
@@ -208,6 +209,18 @@ __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, i
         "l"(map), "r"(x), "r"(y), "r"(smem_addr(bar))
         : "memory");
 }
+
+// Tensor TMA store of a tile from shared memory; parts outside the map are
+// left out.  Completion by bulk groups of the issuing thread.
+__device__ __forceinline__ void tma_store_3d(const CUtensorMap *map, const void *src, int x, int y, int z)
+{
+    asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.tile.bulk_group [%0, {%2, %3, %4}], [%1];" ::"l"(map),
+                 "r"(smem_addr(src)), "r"(x), "r"(y), "r"(z)
+                 : "memory");
+}
+__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
 __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t bytes, uint64_t *bar)
 {
@@ -364,73 +377,62 @@ __device__ __forceinline__ void ring_moments(const real (&f)[NV], const real (&v
 }
 
 // ---------------------------------------------------------------------------
-// One site's update (Eq. LB_evolution_equation, Eq. Eqlambda), all 33
-// velocities unrolled.  sp/sc/sn: shared-memory buffers of rows m-1, m, m+1;
-// col = HALO + tx.  Velocity (k, i) has Cartesian direction i pi / 4, so its
-// moments and equilibrium use the fixed direction cosines; its polar Courant
-// numbers use the row's c_i = cos(i pi/4 - theta_m), s_i = sin(...).
+// One site's FP32 update (Eq. LB_evolution_equation, Eq. Eqlambda), all 33
+// velocities unrolled; returns the new stored reaction variable.  f: the site's
+// own values; lst: its stored reaction variable y = 1 - lambda.  Velocity (k,
+// i) has Cartesian direction i pi / 4, so its moments and equilibrium use the
+// fixed direction cosines; its polar Courant numbers use the row's c_i =
+// cos(i pi/4 - theta_m), s_i = sin(...), i < 4.  radial(q, i) and theta(q, i)
+// give the upwind neighbours of velocity q in direction i, lam_radial(inner)
+// and lam_theta(below) those of y; put(q, v) takes the new f of velocity q.
+//
+// The 8 velocities of a ring go through each operation together: 8 independent
+// instructions in a row, which with two warps per SM quarter is what hides
+// their latency (velocity by velocity the same update takes 18 % more cycles
+// from shared memory to shared memory).
 // ---------------------------------------------------------------------------
-template <typename real, int WP, bool REREAD = false, int LAMOFF = NV * WP, bool DIR_OUTER = false>
-__device__ __forceinline__ void site_update(const StepArgs<real> &A, const StepConsts<real> &C,
-                                            const real *__restrict__ sp,
-                                            const real *__restrict__ sc,
-                                            const real *__restrict__ sn, int col, int j, int m,
-                                            real inv_r, const real (&cs)[8], const real (&sn8)[8])
+template <typename Radial, typename Theta, typename Put, typename LamR, typename LamT>
+__device__ __forceinline__ float site_update(const StepConsts<float> &C, const float (&f)[NV], float lst, int ld,
+                                                int j, int m, float inv_r, const float (&cs)[4],
+                                                const float (&sn4)[4], Radial radial, Theta theta, Put put,
+                                                LamR lam_radial, LamT lam_theta)
 {
-    using O = Op<real>;
-    const real H = real(0.70710678118654752440);  // cos(pi/4)
-    const real one = real(1), half = real(0.5);
-    // the site's stores stay inside its instance's planes
-    if (!DBM_DEBUG_CHECK(j >= 0 && j < A.nr && A.nr <= A.ld && m >= 0 && m < A.ntheta, A.status)) return;
-
-    // --- a1: load the site's 33 f and lambda -------------------------------
-    real f[NV];
-#pragma unroll
-    for (int q = 0; q < NV; ++q) f[q] = sc[q * WP + col];
-    constexpr bool kY = LamStore<real>::complement;
-    const real lst = sc[LAMOFF + col];  // stored: lambda, or y = 1 - lambda
-    const real lam = kY ? O::sub(one, lst) : lst;
+    using O = Op<float>;
+    const float H = 0.70710678118654752440f;
+    const float lam = O::sub(1.f, lst);
 
     // --- a2: moments, ring by ring (Cartesian components) ------------------
     //     rho = sum f, rho u = sum f v, e2 = sum f v^2, T = (e2/rho - u^2)/2
-    real rho, jx, jy, e2;
-    ring_moments<real>(f, C.v, C.v2, rho, jx, jy, e2);
-    const real inv_rho = O::rcp(rho);
-    const real ux = O::mul(jx, inv_rho), uy = O::mul(jy, inv_rho);
-    const real u2 = O::fma(ux, ux, O::mul(uy, uy));
-    const real T = O::mul(half, O::sub(O::mul(e2, inv_rho), u2));
-    const real inv_T = O::rcp(T);
+    float rho, jx, jy, e2;
+    ring_moments<float>(f, C.v, C.v2, rho, jx, jy, e2);
+    const float inv_rho = O::rcp(rho);
+    const float ux = O::mul(jx, inv_rho), uy = O::mul(jy, inv_rho);
+    const float u2 = O::fma(ux, ux, O::mul(uy, uy));
+    const float T = O::mul(0.5f, O::sub(O::mul(e2, inv_rho), u2));
+    const float inv_T = O::rcp(T);
 
     // --- a3: weights F_k(T), F_0 = 1 - 8 sum F_k ---------------------------
-    real F[4];
-    real Fsum = real(0);
+    float F[4];
+    float Fsum = 0.f;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         F[k] = O::mul(T, O::fma(T, O::fma(T, O::fma(T, C.Fc[k][3], C.Fc[k][2]), C.Fc[k][1]), C.Fc[k][0]));
         Fsum = O::add(Fsum, F[k]);
     }
-    const real F0 = O::fma(real(-8), Fsum, one);
+    const float F0 = O::fma(-8.f, Fsum, 1.f);
 
     // --- a4 coefficients: f^eq = rho F_k [A0 + A1 xi + A2 xi^2 + xi^3/6 + xi^4/24],
-    //     xi = v.u / T ---------------------------------------------------------
-    const real hh = O::mul(O::mul(half, u2), inv_T);
-    const real A1 = O::sub(one, hh);
-    const real A0 = O::fma(O::mul(half, hh), hh, A1);
-    const real A2 = O::mul(half, A1);
-    const real wx = O::mul(ux, inv_T), wy = O::mul(uy, inv_T);
-    real w[8];
-    w[0] = wx;
-    w[2] = wy;
-    w[1] = O::mul(H, O::add(wx, wy));
-    w[3] = O::mul(H, O::sub(wy, wx));
-    w[4] = -w[0];
-    w[5] = -w[1];
-    w[6] = -w[2];
-    w[7] = -w[3];
+    //     xi = v.u / T = v_k w_i; opposite directions have -w ------------------
+    const float hh = O::mul(O::mul(0.5f, u2), inv_T);
+    const float A1 = O::sub(1.f, hh);
+    const float A0 = O::fma(O::mul(0.5f, hh), hh, A1);
+    const float A2 = O::mul(0.5f, A1);
+    const float wx = O::mul(ux, inv_T), wy = O::mul(uy, inv_T);
+    const float w[4] = {wx, O::mul(H, O::add(wx, wy)), wy, O::mul(H, O::sub(wy, wx))};
 
     // --- a5: Cochran rate with ignition gate; exact lambda step (a9) -------
-    const real P = O::mul(rho, T);
-    real a = real(0), b = real(0);
+    const float P = O::mul(rho, T);
+    float a = 0.f, b = 0.f;
     if (T > C.T_th) {
         if (C.general_pow) {
             a = O::mul(C.omega1, pow_(P, C.m_exp));
@@ -440,184 +442,152 @@ __device__ __forceinline__ void site_update(const StepArgs<real> &A, const StepC
             b = O::mul(C.omega2, P);
         }
     }
-    const real om = kY ? lst : O::sub(one, lam);  // 1 - lambda
-    const real g = O::fma(b, lam, a);  // a + b lam
-    real R = O::mul(om, g);
-    const real sab = O::add(a, b);
-    real dlam = real(0);
-    if (sab > real(0)) {
+    const float g = O::fma(b, lam, a);  // a + b lam
+    float R = O::mul(lst, g);
+    const float sab = O::add(a, b);
+    float dlam = 0.f;
+    if (sab > 0.f) {
         // lam+ - lam = (1-lam)(a+b lam)(E-1) / [(a+b) + (a+b lam)(E-1)], E = e^{(a+b)dt}
-        const real em1 = expm1_(O::mul(sab, C.dt));
-        dlam = O::mul(O::mul(O::mul(om, g), em1), O::rcp(O::fma(g, em1, sab)));
+        const float em1 = expm1_(O::mul(sab, C.dt));
+        dlam = O::mul(O::mul(O::mul(lst, g), em1), O::rcp(O::fma(g, em1, sab)));
     }
     if (C.reaction_energy) R = O::mul(dlam, C.inv_dt);
 
     // --- a6+a7 coefficients: f_new = poly(xi) (beta_k - gamma_k xi) + ... ---
     //     M = f^eq ((v-u)^2 - 2T) / (2T^2) Q R with (v-u)^2 = v_k^2 + u^2 - 2 T xi
-    const real dtQR = O::mul(C.dt, O::mul(C.Q, R));
-    const real half_inv_T2 = O::mul(O::mul(half, inv_T), inv_T);
-    const real gam = O::mul(dtQR, inv_T);
-    const real u2m2T = O::fma(real(-2), T, u2);
-    const real beta0 = O::mul(O::mul(rho, F0), O::fma(O::mul(dtQR, u2m2T), half_inv_T2, C.one_m_decay));
+    const float dtQR = O::mul(C.dt, O::mul(C.Q, R));
+    const float half_inv_T2 = O::mul(O::mul(0.5f, inv_T), inv_T);
+    const float gam = O::mul(dtQR, inv_T);
+    const float u2m2T = O::fma(-2.f, T, u2);
+    const float beta0 = O::mul(O::mul(rho, F0), O::fma(O::mul(dtQR, u2m2T), half_inv_T2, C.one_m_decay));
+    put(0, O::fma(A0, beta0, O::mul(C.decay, f[0])));
 
-    // --- a8: per-direction Courant magnitudes and upwind neighbours --------
-    const int to_prev = (int)(sp - sc), to_next = (int)(sn - sc);
-    const bool wrap_prev = C.sector && m == 0;             // row -1 = last row, i -> i+1
-    const bool wrap_next = C.sector && m == A.ntheta - 1;  // row ntheta = row 0, i -> i-1
-    // direction i: |C_r| / v_k, |C_theta| / v_k, their sum, and the shared-memory
-    // offsets of the upwind neighbours in r and theta (false: a debug check failed)
-    auto geom = [&](int i, real &ar, real &at, real &sa, int &rn, int &tn) -> bool {
-        ar = O::mul(fabs(cs[i]), C.cr_scale);
-        at = O::mul(O::mul(fabs(sn8[i]), C.ct_scale), inv_r);
-        sa = O::add(ar, at);
-        int o = cs[i] >= real(0) ? -1 : 1;  // C_r >= 0: backward difference
-        if (j == 0 && o < 0) {
-            // inner ghost: zero-gradient; the disc centre in a sector (same
-            // site, i -> i+4); on a full disc the site across the centre,
-            // which fill_centre_ghost put in the halo column before col
-            o = C.centre == 1 ? (((i + 4) & 7) - i) * WP : (C.centre == 2 ? -1 : 0);
-        } else if (j == A.nr - 1 && o > 0) {
-            o = 0;  // zero-gradient outer ghost
-        }
-        rn = col + o;
-        if (sn8[i] >= real(0))  // C_theta >= 0: row m-1
-            tn = col + to_prev + (wrap_prev ? (((i + 1) & 7) - i) * WP : 0);
-        else
-            tn = col + to_next + (wrap_next ? (((i + 7) & 7) - i) * WP : 0);
-#ifdef DBM_DEBUG
-        // velocity planes q = 1 + i .. 25 + i of direction i: neighbour
-        // reads stay inside the 33 planes of their row buffer
-        const int tr = tn - (sn8[i] >= real(0) ? to_prev : to_next);
-        const bool ok = (1 + i) * WP + rn >= 0 && (25 + i) * WP + rn < NV * WP &&
-                        (1 + i) * WP + tr >= 0 && (25 + i) * WP + tr < NV * WP;
-        return DBM_DEBUG_CHECK(ok, A.status);
-#else
-        return true;
-#endif
-    };
+    // --- a8: |C_r| / v_k, |C_theta| / v_k and their sum, once per opposite pair
+    //     (the trig table's entry i + 4 is the exact negation of entry i) ------
+    float ar[4], at[4], sa[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        ar[i] = O::mul(fabsf(cs[i]), C.cr_scale);
+        at[i] = O::mul(O::mul(fabsf(sn4[i]), C.ct_scale), inv_r);
+        sa[i] = O::add(ar[i], at[i]);
+    }
 
-    // --- a7 + a11: update all velocities and store ------------------------
+    // --- a7 + a11: update all velocities -----------------------------------
     //     f_new = f^eq (1 - E + dt M/f^eq) + (E - |C_r| - |C_th|) f
     //             + |C_r| f(upwind r) + |C_th| f(upwind theta)
     //     with f^eq (1 - E + dt M / f^eq) = poly(xi) (beta_k - gamma_k xi) in ring k
-    real *out = A.f_out + (long long)m * A.ld + j;
-    out[0] = O::fma(A0, beta0, O::mul(C.decay, REREAD ? sc[col] : f[0]));
-    if constexpr (!DIR_OUTER) {
-        // Ring by ring with the geometry of all 8 directions held: the
-        // single-instance kernels.
-        real ar[8], at[8], sa[8];
-        int rn[8], tn[8];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            // as geom(i, ...), written out: the compiler schedules this form better
-            ar[i] = O::mul(fabs(cs[i]), C.cr_scale);
-            at[i] = O::mul(O::mul(fabs(sn8[i]), C.ct_scale), inv_r);
-            sa[i] = O::add(ar[i], at[i]);
-            int o = cs[i] >= real(0) ? -1 : 1;  // C_r >= 0: backward difference
-            if (j == 0 && o < 0) {
-                o = C.centre == 1 ? (((i + 4) & 7) - i) * WP : (C.centre == 2 ? -1 : 0);
-            } else if (j == A.nr - 1 && o > 0) {
-                o = 0;  // zero-gradient outer ghost
-            }
-            rn[i] = col + o;
-            if (sn8[i] >= real(0))  // C_theta >= 0: row m-1
-                tn[i] = col + to_prev + (wrap_prev ? (((i + 1) & 7) - i) * WP : 0);
-            else
-                tn[i] = col + to_next + (wrap_next ? (((i + 7) & 7) - i) * WP : 0);
-#ifdef DBM_DEBUG
-            {
-                // velocity planes q = 1 + i .. 25 + i of direction i: neighbour
-                // reads stay inside the 33 planes of their row buffer
-                const int tr = tn[i] - (sn8[i] >= real(0) ? to_prev : to_next);
-                const bool ok = (1 + i) * WP + rn[i] >= 0 && (25 + i) * WP + rn[i] < NV * WP &&
-                                (1 + i) * WP + tr >= 0 && (25 + i) * WP + tr < NV * WP;
-                if (!DBM_DEBUG_CHECK(ok, A.status)) return;
-            }
-#endif
-        }
+    for (int k = 0; k < 4; ++k) {
+        const float vk = C.v[k];
+        const float rF = O::mul(rho, F[k]);
+        const float beta = O::mul(rF, O::fma(O::mul(dtQR, O::add(C.v2[k], u2m2T)), half_inv_T2, C.one_m_decay));
+        const float gamma = O::mul(rF, gam);
+        const int q = 1 + 8 * k;
+        float xi[8], pl[8], t[8], adv[8], keep[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const real vk = C.v[k];
-            const real rF = O::mul(rho, F[k]);
-            const real beta = O::mul(rF, O::fma(O::mul(dtQR, O::add(C.v2[k], u2m2T)), half_inv_T2, C.one_m_decay));
-            const real gamma = O::mul(rF, gam);
-            // one velocity given its xi and the equilibrium polynomial at xi
-            auto update_one = [&](int i, real xi, real poly) {
-                const int q = 1 + 8 * k + i;
-                real t = O::mul(poly, O::fma(-gamma, xi, beta));
-                // REREAD: take f from shared memory again instead of holding all
-                // 33 values in registers across the moment pass (fewer registers)
-                const real fq = REREAD ? sc[q * WP + col] : f[q];
-                t = O::fma(O::fma(-vk, sa[i], C.decay), fq, t);
-                const real adv = O::fma(ar[i], sc[q * WP + rn[i]], O::mul(at[i], sc[q * WP + tn[i]]));
-                t = O::fma(vk, adv, t);
-                out[(long long)q * A.plane] = t;
-            };
+        for (int i = 0; i < 8; ++i) adv[i] = O::mul(at[i & 3], theta(q + i, i));
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const real xi = O::mul(vk, w[i]);
-                update_one(i, xi, O::fma(xi, O::fma(xi, O::fma(xi, O::fma(xi, real(1.0 / 24.0), real(1.0 / 6.0)), A2), A1), A0));
-            }
-        }
-    } else {
-        // DIR_OUTER (batched launches, which hold each instance's
-        // constants in registers): direction by direction, so that only one
-        // direction's geometry is live at a time.  Each velocity's arithmetic
-        // is the ring-by-ring one, operation for operation: same bits.
-        real beta[4], gamma[4];
+        for (int i = 0; i < 8; ++i) adv[i] = O::fma(ar[i & 3], radial(q + i, i), adv[i]);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const real rF = O::mul(rho, F[k]);
-            beta[k] = O::mul(rF, O::fma(O::mul(dtQR, O::add(C.v2[k], u2m2T)), half_inv_T2, C.one_m_decay));
-            gamma[k] = O::mul(rF, gam);
-        }
+        for (int i = 0; i < 4; ++i) xi[i] = O::mul(vk, w[i]);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            real ar, at, sa;
-            int rn, tn;
-            if (!geom(i, ar, at, sa, rn, tn)) return;
+        for (int i = 0; i < 4; ++i) xi[i + 4] = -xi[i];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int q = 1 + 8 * k + i;
-                const real vk = C.v[k];
-                const real xi = O::mul(vk, w[i]);
-                const real poly =
-                    O::fma(xi, O::fma(xi, O::fma(xi, O::fma(xi, real(1.0 / 24.0), real(1.0 / 6.0)), A2), A1), A0);
-                real t = O::mul(poly, O::fma(-gamma[k], xi, beta[k]));
-                const real fq = REREAD ? sc[q * WP + col] : f[q];
-                t = O::fma(O::fma(-vk, sa, C.decay), fq, t);
-                const real adv = O::fma(ar, sc[q * WP + rn], O::mul(at, sc[q * WP + tn]));
-                t = O::fma(vk, adv, t);
-                out[(long long)q * A.plane] = t;
-            }
-        }
+        for (int i = 0; i < 8; ++i) pl[i] = O::fma(xi[i], float(1.0 / 24.0), float(1.0 / 6.0));
+#pragma unroll
+        for (int i = 0; i < 8; ++i) pl[i] = O::fma(xi[i], pl[i], A2);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) pl[i] = O::fma(xi[i], pl[i], A1);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) pl[i] = O::fma(xi[i], pl[i], A0);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) t[i] = O::fma(-gamma, xi[i], beta);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) keep[i] = O::fma(-vk, sa[i], C.decay);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) t[i] = O::mul(pl[i], t[i]);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) t[i] = O::fma(keep[i & 3], f[q + i], t[i]);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) put(q + i, O::fma(vk, adv[i], t[i]));
     }
 
     // --- a9 + a10: lambda = exact reaction step + upwind transport ---------
-    const real cth = cs[0], sth = -sn8[0];  // cos(theta_m), sin(theta_m)
-    const real ur = O::fma(ux, cth, O::mul(uy, sth));
-    const real uth = O::fma(uy, cth, -O::mul(ux, sth));
-    int orr = ur >= real(0) ? -1 : 1;
-    if ((j == 0 && orr < 0 && C.centre != 2) || (j == A.nr - 1 && orr > 0)) orr = 0;
-    // transport acts on the stored variable alike (y - y_nb = lambda_nb - lambda);
-    // the reaction step adds dlam to lambda, so it is taken off y
-    if (!DBM_DEBUG_CHECK(col + orr >= 0 && col + orr < WP, A.status)) return;
-    const real lr = sc[LAMOFF + col + orr];
-    const real lt = (uth >= real(0) ? sp : sn)[LAMOFF + col];
-    const real tr = O::mul(O::mul(fabs(ur), C.cr_scale), O::sub(lst, lr));
-    const real tt = O::mul(O::mul(O::mul(fabs(uth), C.ct_scale), inv_r), O::sub(lst, lt));
-    // y - dlam - tr - tt summed exactly, then rounded without bias
+    const float cth = cs[0], sth = -sn4[0];
+    const float ur = O::fma(ux, cth, O::mul(uy, sth));
+    const float uth = O::fma(uy, cth, -O::mul(ux, sth));
+    const float tr = O::mul(O::mul(fabsf(ur), C.cr_scale), O::sub(lst, lam_radial(ur >= 0.f)));
+    const float tt = O::mul(O::mul(O::mul(fabsf(uth), C.ct_scale), inv_r), O::sub(lst, lam_theta(uth >= 0.f)));
+    // transport acts on the stored variable alike (y - y_nb = lambda_nb - lambda),
+    // the reaction step's dlam is taken off y: y - dlam - tr - tt summed exactly,
+    // then rounded without bias
     float sum, err, e;
     two_sum_f(lst, -dlam, sum, err);
     two_sum_f(sum, -tr, sum, e);
     err = __fadd_rn(err, e);
     two_sum_f(sum, -tt, sum, e);
     err = __fadd_rn(err, e);
-    const uint32_t site = (uint32_t)m * (uint32_t)A.ld + (uint32_t)j;
+    const uint32_t site = (uint32_t)m * (uint32_t)ld + (uint32_t)j;
     const float u = (float)(hash32(site * 0x9e3779b9u ^ __float_as_uint(lst)) >> 8) * 0x1p-24f;
-    real ln = round_stochastic_unit(sum, err, u);
-    ln = fmin(fmax(ln, real(0)), real(1));
-    A.lam_out[(long long)m * A.ld + j] = ln;
+    return fminf(fmaxf(round_stochastic_unit(sum, err, u), 0.f), 1.f);
+}
+
+// Upwind signs of a row: whether direction i's radial (theta) neighbour is the
+// inner (lower) one.  The trig table's entry i + 4 is the negation of entry i.
+__device__ __forceinline__ bool upwind_below(const float (&c)[4], int i)
+{
+    return i < 4 ? c[i & 3] >= 0.f : c[i & 3] <= 0.f;  // C >= 0: backward difference
+}
+
+// The update from row buffers in shared memory: sp/sc/sn hold rows m-1, m, m+1,
+// col is the site's column.  A row's directions share their signs and a site
+// its two radial neighbours, so a neighbour is one select; only a sector's disc
+// centre and first and last row turn the velocity set.
+template <int WP, int LAMOFF, typename Put>
+__device__ __forceinline__ void ring_site_update(const StepArgs<float> &A, const StepConsts<float> &C,
+                                                 const float *__restrict__ sp, const float *__restrict__ sc,
+                                                 const float *__restrict__ sn, int col, int j, int m, float inv_r,
+                                                 const float (&cs)[4], const float (&sn4)[4], bool active, Put put)
+{
+    // the site's stores stay inside its instance's planes
+    if (!DBM_DEBUG_CHECK(j >= 0 && (j < A.nr || !active) && A.nr <= A.ld && m >= 0 && m < A.ntheta, A.status)) return;
+    float f[NV];
+#pragma unroll
+    for (int q = 0; q < NV; ++q) f[q] = sc[q * WP + col];
+    // inner ghost: zero-gradient; on a full disc the site across the centre,
+    // which fill_centre_ghost put in the halo column before col
+    const float *left = sc + col - (j > 0 || C.centre == 2 ? 1 : 0), *right = sc + col + (j < A.nr - 1 ? 1 : 0);
+    const float *prev = sp + col, *next = sn + col;
+    const float *rn[8], *tn[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        rn[i] = upwind_below(cs, i) ? left : right;
+        tn[i] = upwind_below(sn4, i) ? prev : next;
+    }
+    if (C.sector) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            if (C.centre == 1 && j == 0 && upwind_below(cs, i)) rn[i] += (((i + 4) & 7) - i) * WP;  // same site, i -> i+4
+            if (m == 0 && upwind_below(sn4, i)) tn[i] += (((i + 1) & 7) - i) * WP;  // row -1 = last row, i -> i+1
+            if (m == A.ntheta - 1 && !upwind_below(sn4, i)) tn[i] += (((i + 7) & 7) - i) * WP;  // row 0, i -> i-1
+        }
+    }
+#ifdef DBM_DEBUG
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        // velocity planes q = 1 + i .. 25 + i of direction i: neighbour reads
+        // stay inside the 33 planes of their row buffer
+        const int r = (int)(rn[i] - sc), t = (int)(tn[i] - (upwind_below(sn4, i) ? sp : sn));
+        const bool ok = (1 + i) * WP + r >= 0 && (25 + i) * WP + r < NV * WP && (1 + i) * WP + t >= 0 &&
+                        (25 + i) * WP + t < NV * WP;
+        if (!DBM_DEBUG_CHECK(ok, A.status)) return;
+    }
+#endif
+    const float ln = site_update(
+        C, f, sc[LAMOFF + col], A.ld, j, m, inv_r, cs, sn4, [&](int q, int i) { return rn[i][q * WP]; },
+        [&](int q, int i) { return tn[i][q * WP]; }, put, [&](bool inner) { return (inner ? left : right)[LAMOFF]; },
+        [&](bool below) { return (below ? prev : next)[LAMOFF]; });
+    if (active) A.lam_out[(long long)m * A.ld + j] = ln;
 }
 
 }  // namespace dbm
@@ -841,17 +811,19 @@ __device__ __forceinline__ void march(const Work &work, unsigned char *smem_raw,
                     if (ghost) fence_proxy_async_smem();
                 }
             } else if (active && !abort_flag) {
-                real cs[8], sn8[8];
+                real cs[4], sn4[4];
                 const real *rt = A.rowtab + (long long)m * 16;
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
+                for (int i = 0; i < 4; ++i) {
                     cs[i] = rt[i];
-                    sn8[i] = rt[8 + i];
+                    sn4[i] = rt[8 + i];
                 }
                 const bool ghost = C.centre == 2 && j == 0;
                 if (ghost) fill_centre_ghost<real, WP, NV * WP, HALO>(A, sm + (P % NSTAGE) * SLOT, m);
-                site_update<real, WP>(A, C, sm + ((P - 1) % NSTAGE) * SLOT, sm + (P % NSTAGE) * SLOT,
-                                      sm + ((P + 1) % NSTAGE) * SLOT, HALO + tx, j, m, inv_r, cs, sn8);
+                real *out = A.f_out + (long long)m * A.ld + j;
+                ring_site_update<WP, NV * WP>(A, C, sm + ((P - 1) % NSTAGE) * SLOT, sm + (P % NSTAGE) * SLOT,
+                                         sm + ((P + 1) % NSTAGE) * SLOT, HALO + tx, j, m, inv_r, cs, sn4, true,
+                                         [&](int q, float v) { out[(long long)q * A.plane] = v; });
                 if (ghost) fence_proxy_async_smem();
             }
             __syncthreads();
@@ -920,7 +892,7 @@ struct V2Layout {
 // for the slowest.  Positions are released after their last use: after
 // centre P the buffer of P-1, and at an item's last centre also P and P+1.
 // ---------------------------------------------------------------------------
-template <typename real, int W, int NSTAGE, bool REREAD, bool TMAP, typename Work>
+template <typename real, int W, int NSTAGE, bool STAGE, bool TMAP, typename Work>
 __device__ __forceinline__ void march2(const Work &work, unsigned char *smem_raw,
                                        StepArgs<real> *sargs2)
 {
@@ -940,7 +912,8 @@ __device__ __forceinline__ void march2(const Work &work, unsigned char *smem_raw
     static_assert((RTOFF * sizeof(real)) % 16 == 0, "trig row must be 16-byte aligned");
 
     real *sm = reinterpret_cast<real *>(smem_raw);
-    uint64_t *full = reinterpret_cast<uint64_t *>(smem_raw + sizeof(real) * NSTAGE * SLOT);
+    static_assert(!STAGE || (TMAP && sizeof(real) == 4), "staged rows are FP32, stored through a tensor map");
+    uint64_t *full = reinterpret_cast<uint64_t *>(smem_raw + sizeof(real) * (NSTAGE * SLOT + (STAGE ? NV * W : 0)));
     uint64_t *empty = full + NSTAGE;
     __shared__ int abort_flag;
     __shared__ int issued_total;
@@ -1068,7 +1041,9 @@ __device__ __forceinline__ void march2(const Work &work, unsigned char *smem_raw
         int parity = 0;
         bool ok = true;
         // One work item: rows [mb, me) of the strip starting at radial site j0.
-        auto run_item = [&](const StepArgs<real> &A, const StepConsts<real> &C, int j0, int mb, int me) {
+        real *stage = sm + NSTAGE * SLOT + warp * (NV * 32);  // STAGE: this warp's outgoing row
+        auto run_item = [&](const StepArgs<real> &A, const StepConsts<real> &C, const CUtensorMap *out_map, int j0,
+                            int mb, int me) {
             const int L = me - mb;
             const int j = j0 + tx;
             const bool active = j < A.nr;
@@ -1095,20 +1070,38 @@ __device__ __forceinline__ void march2(const Work &work, unsigned char *smem_raw
                                                          sm + ((P + 1) % NSTAGE) * SLOT, j0, tx, mb + c - 1,
                                                          sc + RTOFF);
                     if (ghost) fence_proxy_async_smem();
-                } else if (active) {
-                    real cs[8], sn8[8];
+                } else if (active || STAGE) {
+                    real cs[4], sn4[4];
                     const real *rt = sc + RTOFF;
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) {
+                    for (int i = 0; i < 4; ++i) {
                         cs[i] = rt[i];
-                        sn8[i] = rt[8 + i];
+                        sn4[i] = rt[8 + i];
                     }
                     const bool ghost = C.centre == 2 && j == 0;
                     if (ghost)
                         fill_centre_ghost<real, WP, LAMOFF, HALO>(A, sm + (P % NSTAGE) * SLOT, mb + c - 1);
-                    site_update<real, WP, REREAD, LAMOFF, Work::kCopyArgs>(A, C, sm + ((P - 1) % NSTAGE) * SLOT, sc,
-                                                  sm + ((P + 1) % NSTAGE) * SLOT, HALO + tx, j,
-                                                  mb + c - 1, inv_r, cs, sn8);
+                    const real *sp = sm + ((P - 1) % NSTAGE) * SLOT, *sn = sm + ((P + 1) % NSTAGE) * SLOT;
+                    if constexpr (STAGE) {
+                        ring_site_update<WP, LAMOFF>(A, C, sp, sc, sn, HALO + tx, j, mb + c - 1, inv_r, cs, sn4, active,
+                                                [&](int q, float v) {
+                                                    if (q == 0) {  // the store before has read the staging row
+                                                        if (lane == 0) bulk_wait_read();
+                                                        __syncwarp();
+                                                    }
+                                                    stage[q * 32 + lane] = v;
+                                                });
+                        fence_proxy_async_smem();
+                        __syncwarp();
+                        if (lane == 0 && j < A.nr) {
+                            tma_store_3d(out_map, stage, j, mb + c - 1, 0);
+                            bulk_commit();
+                        }
+                    } else {
+                        real *out = A.f_out + (long long)(mb + c - 1) * A.ld + j;
+                        ring_site_update<WP, LAMOFF>(A, C, sp, sc, sn, HALO + tx, j, mb + c - 1, inv_r, cs, sn4, true,
+                                                [&](int q, float v) { out[(long long)q * A.plane] = v; });
+                    }
                     if (ghost) fence_proxy_async_smem();
                 }
                 __syncwarp();
@@ -1136,6 +1129,7 @@ __device__ __forceinline__ void march2(const Work &work, unsigned char *smem_raw
                     reinterpret_cast<int *>(dst)[q] = reinterpret_cast<const int *>(ga)[q];
                 named_bar_sync(1, W);
                 parity ^= 1;
+                if (STAGE && lane == 0) fence_tensormap_acquire(&ga->tm_out);
                 // FP32: the item's pointers and sizes from there, and its
                 // constants from the batch constant table, into registers for
                 // the item (a single instance reads its constants from the
@@ -1148,14 +1142,15 @@ __device__ __forceinline__ void march2(const Work &work, unsigned char *smem_raw
                 if constexpr (sizeof(real) == 4) {
                     const StepArgs<real> Areg = *dst;
                     const StepConsts<real> Creg = C;
-                    run_item(Areg, Creg, j0, mb, me);
+                    run_item(Areg, Creg, &ga->tm_out, j0, mb, me);
                 } else {
-                    run_item(*dst, C, j0, mb, me);
+                    run_item(*dst, C, &ga->tm_out, j0, mb, me);
                 }
             } else {
-                run_item(*ga, ga->c, j0, mb, me);
+                run_item(*ga, ga->c, &ga->tm_out, j0, mb, me);
             }
         }
+        if (STAGE && lane == 0) bulk_wait_all();  // rows written, and read out of shared memory
     }
     __syncthreads();
     if (abort_flag && tx == 0) {
@@ -1166,27 +1161,27 @@ __device__ __forceinline__ void march2(const Work &work, unsigned char *smem_raw
     }
 }
 
-template <typename real, int W, int NSTAGE, bool REREAD, int MINB, bool TMAP>
+template <typename real, int W, int NSTAGE, bool STAGE, int MINB, bool TMAP>
 __global__ void __launch_bounds__(W + 32, MINB) step_kernel_v2(const __grid_constant__ StepArgs<real> A)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     SingleWork<real, W> work{&A};
-    march2<real, W, NSTAGE, REREAD, TMAP>(work, smem_raw, nullptr);
+    march2<real, W, NSTAGE, STAGE, TMAP>(work, smem_raw, nullptr);
 }
 
-template <typename real, int W, int NSTAGE, bool REREAD, int MINB, bool TMAP>
+template <typename real, int W, int NSTAGE, bool STAGE, int MINB, bool TMAP>
 __global__ void __launch_bounds__(W + 32, MINB) batch_step_kernel_v2(const __grid_constant__ BatchArgs<real> B)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ __align__(64) StepArgs<real> sargs2[2];
     BatchWork<real, W> work{B.slots, B.items, *B.n_items, *B.T + B.s};
-    march2<real, W, NSTAGE, REREAD, TMAP>(work, smem_raw, sargs2);
+    march2<real, W, NSTAGE, STAGE, TMAP>(work, smem_raw, sargs2);
 }
 
-template <typename real, int W, int NSTAGE>
+template <typename real, int W, int NSTAGE, bool STAGE>
 constexpr int smem_bytes_v2()
 {
-    return (int)(sizeof(real) * NSTAGE * V2Layout<real, W>::slot + 16 * NSTAGE);
+    return (int)(sizeof(real) * (NSTAGE * V2Layout<real, W>::slot + (STAGE ? NV * W : 0)) + 16 * NSTAGE);
 }
 
 // Self-test of the bounded wait every pipeline uses: one CTA waits on an

@@ -29,7 +29,7 @@ template <typename real> int default_variant();
 template <typename real> int fallback_variant();
 template <typename real> cudaError_t kernel_info(int variant, KernelInfo *out);
 template <typename real> cudaError_t launch_step(int variant, const StepArgs<real> &A, int grid, cudaStream_t s);
-// The FP64 step straight from global memory.
+// The step straight from global memory (one simulation).
 cudaError_t launch_direct64(const Direct64Args &D, cudaStream_t s);
 template <typename real> cudaError_t batch_kernel_info(int variant, KernelInfo *out);
 template <typename real>

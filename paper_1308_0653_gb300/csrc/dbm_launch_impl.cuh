@@ -1,6 +1,6 @@
 // Instantiates the kernels of one precision; included once per precision
 // translation unit with DBM_REAL and the variant list DBM_VARIANTS(X) defined,
-// X(id, version, W, NSTAGE, REREAD, MIN_BLOCKS_PER_SM), DBM_DEFAULT_VARIANT and
+// X(id, version, W, NSTAGE, STAGE, MIN_BLOCKS_PER_SM), DBM_DEFAULT_VARIANT and
 // DBM_FALLBACK_VARIANT (the default when tensor maps are unavailable).
 // version 1: CTA-wide row barrier; 2: producer warp, per-array bulk copies;
 // 3: producer warp, tensor-map TMA tiles.
@@ -32,10 +32,10 @@ cudaError_t upload_batch_consts<DBM_REAL>(int first, const StepConsts<DBM_REAL> 
 
 namespace {
 
-template <int VER, int W, int NS, bool RR, int MB> struct Variant;
+template <int VER, int W, int NS, bool ST, int MB> struct Variant;
 
-template <int W, int NS, bool RR, int MB>
-struct Variant<1, W, NS, RR, MB> {
+template <int W, int NS, bool ST, int MB>
+struct Variant<1, W, NS, ST, MB> {
     static constexpr int kThreads = W;
     static constexpr int kSmem =
         (int)(sizeof(DBM_REAL) * NS * NARR * (W + 2 * Halo<DBM_REAL>::value) + 8 * NS);
@@ -53,29 +53,29 @@ struct Variant<1, W, NS, RR, MB> {
     }
 };
 
-template <int W, int NS, bool RR, int MB, bool TM>
+template <int W, int NS, bool ST, int MB, bool TM>
 struct VariantV2 {
     static constexpr int kThreads = W + 32;
-    static constexpr int kSmem = smem_bytes_v2<DBM_REAL, W, NS>();
-    static void *single() { return (void *)step_kernel_v2<DBM_REAL, W, NS, RR, MB, TM>; }
-    static void *batch() { return (void *)batch_step_kernel_v2<DBM_REAL, W, NS, RR, MB, TM>; }
+    static constexpr int kSmem = smem_bytes_v2<DBM_REAL, W, NS, ST>();
+    static void *single() { return (void *)step_kernel_v2<DBM_REAL, W, NS, ST, MB, TM>; }
+    static void *batch() { return (void *)batch_step_kernel_v2<DBM_REAL, W, NS, ST, MB, TM>; }
     static cudaError_t run(const StepArgs<DBM_REAL> &A, int g, cudaStream_t s)
     {
-        step_kernel_v2<DBM_REAL, W, NS, RR, MB, TM><<<g, kThreads, kSmem, s>>>(A);
+        step_kernel_v2<DBM_REAL, W, NS, ST, MB, TM><<<g, kThreads, kSmem, s>>>(A);
         return cudaGetLastError();
     }
     static cudaError_t run_batch(const BatchArgs<DBM_REAL> &B, int g, cudaStream_t s)
     {
-        batch_step_kernel_v2<DBM_REAL, W, NS, RR, MB, TM><<<g, kThreads, kSmem, s>>>(B);
+        batch_step_kernel_v2<DBM_REAL, W, NS, ST, MB, TM><<<g, kThreads, kSmem, s>>>(B);
         return cudaGetLastError();
     }
 };
 
-template <int W, int NS, bool RR, int MB>
-struct Variant<2, W, NS, RR, MB> : VariantV2<W, NS, RR, MB, false> {};
+template <int W, int NS, bool ST, int MB>
+struct Variant<2, W, NS, ST, MB> : VariantV2<W, NS, ST, MB, false> {};
 
-template <int W, int NS, bool RR, int MB>
-struct Variant<3, W, NS, RR, MB> : VariantV2<W, NS, RR, MB, true> {};
+template <int W, int NS, bool ST, int MB>
+struct Variant<3, W, NS, ST, MB> : VariantV2<W, NS, ST, MB, true> {};
 
 template <typename V>
 cudaError_t info_of(void *fn, int ver, int W, int NS, KernelInfo *out)
@@ -100,7 +100,7 @@ cudaError_t info_of(void *fn, int ver, int W, int NS, KernelInfo *out)
 template <> int num_variants<DBM_REAL>()
 {
     int n = 0;
-#define X(id, ver, W, NS, RR, MB) n = n > id ? n : id;
+#define X(id, ver, W, NS, ST, MB) n = n > id ? n : id;
     DBM_VARIANTS(X)
 #undef X
     return n;
@@ -113,8 +113,8 @@ template <>
 cudaError_t kernel_info<DBM_REAL>(int variant, KernelInfo *out)
 {
     switch (variant) {
-#define X(id, ver, W, NS, RR, MB) \
-    case id: return info_of<Variant<ver, W, NS, RR, MB>>(Variant<ver, W, NS, RR, MB>::single(), ver, W, NS, out);
+#define X(id, ver, W, NS, ST, MB) \
+    case id: return info_of<Variant<ver, W, NS, ST, MB>>(Variant<ver, W, NS, ST, MB>::single(), ver, W, NS, out);
         DBM_VARIANTS(X)
 #undef X
     default: return cudaErrorInvalidValue;
@@ -125,8 +125,8 @@ template <>
 cudaError_t batch_kernel_info<DBM_REAL>(int variant, KernelInfo *out)
 {
     switch (variant) {
-#define X(id, ver, W, NS, RR, MB) \
-    case id: return info_of<Variant<ver, W, NS, RR, MB>>(Variant<ver, W, NS, RR, MB>::batch(), ver, W, NS, out);
+#define X(id, ver, W, NS, ST, MB) \
+    case id: return info_of<Variant<ver, W, NS, ST, MB>>(Variant<ver, W, NS, ST, MB>::batch(), ver, W, NS, out);
         DBM_VARIANTS(X)
 #undef X
     default: return cudaErrorInvalidValue;
@@ -137,8 +137,8 @@ template <>
 cudaError_t launch_step<DBM_REAL>(int variant, const StepArgs<DBM_REAL> &A, int grid, cudaStream_t s)
 {
     switch (variant) {
-#define X(id, ver, W, NS, RR, MB) \
-    case id: return Variant<ver, W, NS, RR, MB>::run(A, grid, s);
+#define X(id, ver, W, NS, ST, MB) \
+    case id: return Variant<ver, W, NS, ST, MB>::run(A, grid, s);
         DBM_VARIANTS(X)
 #undef X
     default: return cudaErrorInvalidValue;
@@ -149,8 +149,8 @@ template <>
 cudaError_t launch_batch_step<DBM_REAL>(int variant, const BatchArgs<DBM_REAL> &B, int grid, cudaStream_t s)
 {
     switch (variant) {
-#define X(id, ver, W, NS, RR, MB) \
-    case id: return Variant<ver, W, NS, RR, MB>::run_batch(B, grid, s);
+#define X(id, ver, W, NS, ST, MB) \
+    case id: return Variant<ver, W, NS, ST, MB>::run_batch(B, grid, s);
         DBM_VARIANTS(X)
 #undef X
     default: return cudaErrorInvalidValue;
