@@ -170,6 +170,7 @@ void row_angles(const dbm_params &p, int m, double c[8], double s[8])
 // bit) elsewhere; every other variant always runs its own kernel.
 enum Path {
     PATH_RING,      // the variant's row-ring kernel
+    PATH_DIRECT32,  // FP32, small grids: straight from global memory
     PATH_DIRECT64,  // FP64: straight from global memory
 };
 
@@ -370,6 +371,7 @@ int launch_pass(dbm_t *h, int b, int64_t left, cudaStream_t s, int *took)
     cudaError_t e;
     *took = 1;
     switch (h->path) {
+    case PATH_DIRECT32: e = launch_direct32(h->a32[b], h->nsm, s); break;
     case PATH_DIRECT64: e = launch_direct64(h->d64[b], s); break;
     default:
         e = h->p.precision == DBM_FP64 ? launch_step<double>(h->variant, h->a64[b], h->grid, s)
@@ -460,7 +462,11 @@ void fill_direct64(dbm_t *h)
     }
 }
 
-// The path of the handle's variant.
+// The path of the handle's variant.  FP32 steps straight from global memory up
+// to four waves of 16 warps per SM: there the step is latency, and the ring takes
+// time to fill (64^2 4.1 -> 2.8 us per step, 256^2 6.5 -> 5.3, 512^2, the last
+// size below the line, 14.4 -> 13.6); beyond it the ring's long row copies win
+// (600^2 22.1 against 19.8, 2048^2 238 against 181).
 Path pick_path(const dbm_t *h)
 {
     const dbm_params &p = h->p;
@@ -468,7 +474,7 @@ Path pick_path(const dbm_t *h)
     if (p.precision == DBM_FP64)
         return h->variant == default_variant<double>() && warps <= (1 << 29) ? PATH_DIRECT64 : PATH_RING;
     if (h->variant != default_variant<float>()) return PATH_RING;
-    return PATH_RING;
+    return warps <= 64LL * h->nsm ? PATH_DIRECT32 : PATH_RING;
 }
 
 // Launch shape for a kernel variant: persistent CTAs, one per resident slot,

@@ -15,6 +15,23 @@
 #include "dbm_launch_impl.cuh"
 
 namespace dbm {
+cudaError_t launch_direct32(const StepArgs<float> &A, int nsm, cudaStream_t s)
+{
+    const int log_cols = A.ntheta >= 4 ? 5 : 7, cols = 1 << log_cols, rows = 128 >> log_cols;
+    const long long blocks = (long long)((A.nr + cols - 1) / cols) * ((A.ntheta + rows - 1) / rows);
+    // Three blocks per SM (168 registers) or four (128): a block's time is 0.81
+    // of that with four (64^2, one wave: 2.89 against 3.55 us per step), so what
+    // counts is the number of waves (256^2: 5.43 against 5.26; 320^2: 6.88 against 7.03).
+    const long long waves3 = (blocks + 3 * nsm - 1) / (3 * nsm), waves4 = (blocks + 4 * nsm - 1) / (4 * nsm);
+    if (A.c.sector)
+        direct32_kernel<true, 3><<<(unsigned)blocks, 128, 0, s>>>(A, log_cols);
+    else if (0.81 * waves3 < waves4)
+        direct32_kernel<false, 3><<<(unsigned)blocks, 128, 0, s>>>(A, log_cols);
+    else
+        direct32_kernel<false, 4><<<(unsigned)blocks, 128, 0, s>>>(A, log_cols);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_totals(const double *partials, int nblocks, double *totals, cudaStream_t s)
 {
     totals_kernel<<<1, 256, 0, s>>>(partials, nblocks, totals);

@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include "dbm_device.cuh"
+#include "dbm_direct32.cuh"
 #include "dbm_direct64.cuh"
 
 namespace dbm {
@@ -30,6 +31,7 @@ template <typename real> int fallback_variant();
 template <typename real> cudaError_t kernel_info(int variant, KernelInfo *out);
 template <typename real> cudaError_t launch_step(int variant, const StepArgs<real> &A, int grid, cudaStream_t s);
 // The step straight from global memory (one simulation).
+cudaError_t launch_direct32(const StepArgs<float> &A, int nsm, cudaStream_t s);
 cudaError_t launch_direct64(const Direct64Args &D, cudaStream_t s);
 template <typename real> cudaError_t batch_kernel_info(int variant, KernelInfo *out);
 template <typename real>
