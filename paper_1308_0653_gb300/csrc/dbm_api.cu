@@ -171,6 +171,7 @@ void row_angles(const dbm_params &p, int m, double c[8], double s[8])
 enum Path {
     PATH_RING,      // the variant's row-ring kernel
     PATH_DIRECT32,  // FP32, small grids: straight from global memory
+    PATH_ROW32,     // FP32, one theta row: several steps per pass
     PATH_DIRECT64,  // FP64: straight from global memory
 };
 
@@ -371,6 +372,10 @@ int launch_pass(dbm_t *h, int b, int64_t left, cudaStream_t s, int *took)
     cudaError_t e;
     *took = 1;
     switch (h->path) {
+    case PATH_ROW32:
+        *took = (int)std::min<int64_t>(left, Row32::MAX_STEPS);
+        e = launch_row32(h->a32[b], *took, s);
+        break;
     case PATH_DIRECT32: e = launch_direct32(h->a32[b], h->nsm, s); break;
     case PATH_DIRECT64: e = launch_direct64(h->d64[b], s); break;
     default:
@@ -474,6 +479,7 @@ Path pick_path(const dbm_t *h)
     if (p.precision == DBM_FP64)
         return h->variant == default_variant<double>() && warps <= (1 << 29) ? PATH_DIRECT64 : PATH_RING;
     if (h->variant != default_variant<float>()) return PATH_RING;
+    if (p.ntheta == 1) return PATH_ROW32;
     return warps <= 64LL * h->nsm ? PATH_DIRECT32 : PATH_RING;
 }
 

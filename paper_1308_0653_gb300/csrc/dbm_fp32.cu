@@ -32,6 +32,12 @@ cudaError_t launch_direct32(const StepArgs<float> &A, int nsm, cudaStream_t s)
     return cudaGetLastError();
 }
 
+cudaError_t launch_row32(const StepArgs<float> &A, int steps, cudaStream_t s)
+{
+    row32_kernel<<<(A.nr + Row32::STORED - 1) / Row32::STORED, Row32::WIDTH, 0, s>>>(A, steps);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_totals(const double *partials, int nblocks, double *totals, cudaStream_t s)
 {
     totals_kernel<<<1, 256, 0, s>>>(partials, nblocks, totals);

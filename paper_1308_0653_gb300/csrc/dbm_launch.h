@@ -7,6 +7,7 @@
 #include "dbm_device.cuh"
 #include "dbm_direct32.cuh"
 #include "dbm_direct64.cuh"
+#include "dbm_row32.cuh"
 
 namespace dbm {
 
@@ -32,6 +33,8 @@ template <typename real> cudaError_t kernel_info(int variant, KernelInfo *out);
 template <typename real> cudaError_t launch_step(int variant, const StepArgs<real> &A, int grid, cudaStream_t s);
 // The step straight from global memory (one simulation).
 cudaError_t launch_direct32(const StepArgs<float> &A, int nsm, cudaStream_t s);
+// 1 .. Row32::MAX_STEPS steps of a single theta row.
+cudaError_t launch_row32(const StepArgs<float> &A, int steps, cudaStream_t s);
 cudaError_t launch_direct64(const Direct64Args &D, cudaStream_t s);
 template <typename real> cudaError_t batch_kernel_info(int variant, KernelInfo *out);
 template <typename real>

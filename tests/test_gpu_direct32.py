@@ -1,7 +1,8 @@
-"""The FP32 default's kernel for small grids (straight from global memory) and the
-staged row stores of the row ring against variant 2's row ring, bit for bit, at
-their edges: 32-site warps, four-row and one-row blocks, the line between the
-kernels, ragged widths, every kind of neighbour."""
+"""The FP32 default's other kernels (straight from global memory on small grids,
+several steps per pass on a single theta row) and the staged row stores of the
+row ring against variant 2's row ring, bit for bit, at their edges: 32-site
+warps, four-row blocks, one-row blocks, 96-site row blocks and their 16-step
+passes, the line between the kernels, ragged widths, every kind of neighbour."""
 import numpy as np
 import pytest
 
@@ -35,6 +36,9 @@ def _workload(nr, nth, r_in=0.5, sector=0, r_bc_inner="outflow"):
     (60, 12, dict(r_in=0.0, r_bc_inner="centre"), {}),
     (320, 972, {}, {}), (321, 973, {}, {}),                       # the last grid below the line, one above
     (129, 2500, {}, {}), (255, 1300, {}, {}), (417, 800, {}, {}),  # ring: ragged last strips of 1, 127, 33 sites
+    (15, 1, {}, {}), (96, 1, {}, {}), (97, 1, {}, {}), (1000, 1, {}, {}),                    # single rows
+    (193, 1, dict(sector=1), dict(reaction_energy=1, m=1.5, n=0.7)),
+    (500, 1, dict(sector=1, r_in=0.0, r_bc_inner="centre"), {}),
 ])
 def test_same_bits_as_the_row_ring(nr, nth, shape, options):
     from paper_1308_0653_gb300 import dbm
@@ -43,7 +47,7 @@ def test_same_bits_as_the_row_ring(nr, nth, shape, options):
     for variant in (0, 2):
         sim = dbm.Simulation(dict(w.params, precision="fp32", variant=variant, **options))
         sim.init_state(w.fields)
-        for n in (1, 17, 33, 2):
+        for n in (1, 17, 33, 2):  # passes of 1, 16 + 1, a graph + 1, 2 steps
             sim.step(n)
         f, lam, steps = sim.export_state()
         assert steps == 53 and dbm.dbm_status(sim.h) == dbm.DBM_OK
@@ -53,7 +57,7 @@ def test_same_bits_as_the_row_ring(nr, nth, shape, options):
     assert np.array_equal(got[0][0], got[1][0]) and np.array_equal(got[0][1], got[1][1])
 
 
-@pytest.mark.parametrize("nr,nth", [(40, 4), (700, 700)])
+@pytest.mark.parametrize("nr,nth", [(40, 4), (200, 1), (700, 700)])
 def test_nan_in_lambda_reaches_f(nr, nth):
     """A NaN lambda makes R, and with it the site's f, NaN even where nothing burns."""
     from paper_1308_0653_gb300 import dbm
