@@ -379,6 +379,8 @@ int dbm_batch_plan(int32_t nslots, const int32_t *nr, const int32_t *ntheta, con
 /* Create a batch on caller device memory (256-byte aligned, >=
  * dbm_batch_bytes).  rows_per_item: theta rows per work item (0 = 16; -1 =
  * scaled to each simulation: 16 up to 512 theta rows, 32 up to 1024, else 64).
+ * Items are cut shorter than that while the batch is too small to fill the
+ * persistent CTAs a few times over.
  * Allocates a pinned host staging buffer for the tables and takes max_slots
  * entries of the device's batch constant table (per-slot constants read by
  * the batched kernel from constant memory; DBM_BATCH_CONST_FP32 /
