@@ -459,11 +459,17 @@ void fill_direct64(dbm_t *h)
     const long long chunks = (p.nr + 31) / 32, tasks = chunks * p.ntheta, quarters = 4LL * h->nsm;
     long long full = tasks / quarters * quarters;
     if (4 * (tasks - full) > 2 * quarters) full = tasks;
+    // Beside full tasks the few quarters left over share their SMs' FP64 pipe with
+    // them: one or two to a block where that spreads them over more SMs (20000 x
+    // 1: 68 quarters on 68 SMs instead of 17, 24.4 -> 20.4 us per step).
+    const long long rest = 4 * (tasks - full);
+    const int per_block = full == 0 || rest > 2 * h->nsm ? 4 : rest > h->nsm ? 2 : 1;
     for (int b = 0; b < 2; ++b) {
         h->d64[b].A = h->a64[b];
         h->d64[b].chunks = (int)chunks;
         h->d64[b].full = (int)full;
         h->d64[b].quarters = (int)quarters;
+        h->d64[b].per_block = per_block;
     }
 }
 

@@ -19,7 +19,7 @@ cudaError_t launch_direct64(const Direct64Args &D, cudaStream_t s)
     // up to two waves of warps, each has an SM quarter (nearly) to itself and
     // its loads are not hidden by others
     const long long tasks = (long long)D.chunks * D.A.ntheta;
-    const unsigned blocks = (unsigned)((D.full + 3) / 4 + tasks - D.full);
+    const unsigned blocks = (unsigned)((D.full + 3) / 4 + 4 / D.per_block * (tasks - D.full));
     if (tasks <= 2 * D.quarters)
         direct64_kernel<true><<<blocks, 128, 0, s>>>(D);
     else

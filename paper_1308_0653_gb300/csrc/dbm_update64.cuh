@@ -196,9 +196,15 @@ __device__ __forceinline__ void site_update64(const StepConsts<double> &C, const
     const double b0 = fma(fma(-2.0, T, u2), bs, C.one_m_decay);
 
     double rF[4];
+    if constexpr (G == 4) {
+        const double own = P * fma(T, fma(T, fma(T, C.Fc[mine][3], C.Fc[mine][2]), C.Fc[mine][1]), C.Fc[mine][0]);
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
-        rF[k] = P * fma(T, fma(T, fma(T, C.Fc[k][3], C.Fc[k][2]), C.Fc[k][1]), C.Fc[k][0]);
+        for (int k = 0; k < 4; ++k) rF[k] = __shfl_sync(ALL, own, (lane & 7) + 8 * k);
+    } else {
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            rF[k] = P * fma(T, fma(T, fma(T, C.Fc[k][3], C.Fc[k][2]), C.Fc[k][1]), C.Fc[k][0]);
+    }
     const double rF0 = fma(-8.0, Op64::add(Op64::add(Op64::add(rF[0], rF[1]), rF[2]), rF[3]), rho);
     if (active && (G == 1 || mine == 0)) out[0] = fma(A0, rF0 * b0, C.decay * f0);
 

@@ -34,7 +34,7 @@ def _states(w, **kw):
 
 @pytest.mark.parametrize("nr,nth,kw", [
     (1, 3, {}), (7, 2, {}), (31, 5, {}), (33, 1, {}), (40, 16, {}),            # quarters only
-    (32, 620, {}), (64, 400, {}),                                              # a wave, rest in quarters
+    (32, 620, {}), (32, 668, {}), (64, 400, {}),           # a wave, rest in quarters, 1, 2, 4 to a block
     (100, 230, {}),                                                            # rest too large for quarters
     (257, 151, dict(reaction_energy=1, m=1.5, n=0.7)),                         # more than two waves
     (45, 6, dict(sector=1)), (45, 1, dict(sector=1)), (300, 2, dict(sector=1, r_in=0.0, r_bc_inner="centre")),
