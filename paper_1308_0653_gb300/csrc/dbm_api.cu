@@ -1007,7 +1007,7 @@ static int launch_totals_of(dbm_t *h, int nblocks, cudaStream_t s)
 static int launch_moments_into(dbm_t *h, double *d_out, cudaStream_t s)
 {
     int nblocks = 0;
-    int rc = launch_moments_rows(h, d_out, s, 0, h->p.ntheta, MOMENT_BLOCKS, &nblocks);
+    int rc = launch_moments_rows(h, d_out, s, 0, h->p.ntheta, std::min(MOMENT_BLOCKS, 4 * h->nsm), &nblocks);
     if (rc != DBM_OK) return rc;
     return launch_totals_of(h, nblocks, s);
 }

@@ -1321,14 +1321,17 @@ __global__ void __launch_bounds__(256) init_kernel(const InitArgs<real> A)
 // ring are v_k (cos i pi/4, sin i pi/4)), and all moments are taken from the
 // few ring harmonics.
 // ---------------------------------------------------------------------------
-// f widened to FP64.  Normal floats by shifting their bits: three integer
-// instructions in place of a conversion at the FP64 rate.
+// f widened to FP64.  Floats by shifting their bits, a few integer instructions
+// in place of a conversion at the FP64 rate (subnormals excepted).
 __device__ __forceinline__ double widen(double x) { return x; }
 __device__ __forceinline__ double widen(float x)
 {
-    const uint32_t b = __float_as_uint(x), e = b & 0x7f800000u;
-    if (e == 0u || e == 0x7f800000u) return (double)x;  // zero, subnormal, infinity, NaN
-    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
+    const uint32_t b = __float_as_uint(x), mag = b & 0x7fffffffu;
+    if (mag - 1u < 0x007fffffu) return (double)x;  // subnormal
+    uint32_t hi = (mag >> 3) + 0x38000000u;
+    if (mag >= 0x7f800000u) hi |= 0x38000000u;  // infinity, NaN
+    if (mag == 0u) hi = 0u;
+    return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(b << 29));
 }
 
 // Harmonics of a ring's f: s0 = sum g, (c1, s1) = sum g (cos, sin)(phi),
@@ -1382,8 +1385,25 @@ struct MomArgs {
     int m0, m1;          // theta rows [m0, m1) of this launch
 };
 
+constexpr int MOMENT_THREADS = 256;
+
+// Sums of four values over a warp: component lane / 8 in every lane.  Halving
+// the values while halving the lanes takes 6 additions where a tree per value
+// takes 20 (and FP64 additions are what the reduction costs).
+__device__ __forceinline__ double warp_sum4(const double (&v)[4], int lane)
+{
+    const unsigned ALL = 0xffffffffu;
+    const bool upper = lane & 16, odd = lane & 8;
+    double k0 = upper ? v[2] : v[0], k1 = upper ? v[3] : v[1];
+    k0 += __shfl_xor_sync(ALL, upper ? v[0] : v[2], 16);
+    k1 += __shfl_xor_sync(ALL, upper ? v[1] : v[3], 16);
+    double k = (odd ? k1 : k0) + __shfl_xor_sync(ALL, odd ? k0 : k1, 8);
+    for (int o = 4; o > 0; o >>= 1) k += __shfl_xor_sync(ALL, k, o);
+    return k;
+}
+
 template <typename real>
-__global__ void __launch_bounds__(256) moments_kernel(const MomArgs<real> A)
+__global__ void __launch_bounds__(MOMENT_THREADS) moments_kernel(const MomArgs<real> A)
 {
     const long long N = (long long)A.nr * A.ntheta;
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
@@ -1406,20 +1426,23 @@ __global__ void __launch_bounds__(256) moments_kernel(const MomArgs<real> A)
             const float cth = A.rowtab[(long long)m * 16], sth = -A.rowtab[(long long)m * 16 + 8];
             const float ur = O::fma(ux, cth, O::mul(uy, sth));
             const float uth = O::fma(uy, cth, -O::mul(ux, sth));
-            const double lam = LamStore<float>::to_lambda((double)A.lam[(long long)m * A.ld + j]);
+            // conversions by integer shifts: each would cost an FP64 instruction, and
+            // those, 16 per site with them and 7 without, would take the time
+            const float y = A.lam[(long long)m * A.ld + j];
             if (A.out) {
-                A.out[s] = (double)rho;
-                A.out[N + s] = (double)ur;
-                A.out[2 * N + s] = (double)uth;
-                A.out[3 * N + s] = (double)T;
-                A.out[4 * N + s] = lam;
+                A.out[s] = widen(rho);
+                A.out[N + s] = widen(ur);
+                A.out[2 * N + s] = widen(uth);
+                A.out[3 * N + s] = widen(T);
+                A.out[4 * N + s] = LamStore<float>::to_lambda(widen(y));
             }
-            bad |= !isfinite(rho) || !isfinite(ur) || !isfinite(uth) || !isfinite(T) || !isfinite(lam);
-            const double r = A.r_in + (j + 0.5) * A.dr;  // weight r dr dtheta: dr dtheta applied per block
-            acc[0] += (double)rho * r;
-            acc[1] += (double)jx * r;
-            acc[2] += (double)jy * r;
-            acc[3] += (double)e2 * r;  // rho T + rho u^2 / 2 = (1/2) sum f v^2 for D = 2
+            bad |= !isfinite(rho) || !isfinite(ur) || !isfinite(uth) || !isfinite(T) || !isfinite(y);
+            // weight r dr dtheta: dr dtheta applied per block; j + 1/2 from the bits of 2^52 + j
+            const double r = fma(__hiloint2double(0x43300000, j) - 4503599627370495.5, A.dr, A.r_in);
+            acc[0] = fma(widen(rho), r, acc[0]);
+            acc[1] = fma(widen(jx), r, acc[1]);
+            acc[2] = fma(widen(jy), r, acc[2]);
+            acc[3] = fma(widen(e2), r, acc[3]);  // rho T + rho u^2 / 2 = (1/2) sum f v^2 for D = 2
         }
         const double wa = A.dr * A.dtheta;
         acc[0] *= wa;
@@ -1463,24 +1486,17 @@ __global__ void __launch_bounds__(256) moments_kernel(const MomArgs<real> A)
         acc[3] *= 0.5 * wa;
     }
     if (bad) atomicOr(A.status, ST_NONFINITE);
-    // deterministic block reduction: warp shuffles, then warp 0 over the warps
-    __shared__ double red[4][32];
+    // deterministic block reduction: each warp, then warp 0 over the 8 warps
+    static_assert(MOMENT_THREADS == 256, "one value per lane in the second round");
+    __shared__ double red[4][8];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        double v = acc[c];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if (lane == 0) red[c][wid] = v;
-    }
+    const double v = warp_sum4(acc, lane);
+    if ((lane & 7) == 0) red[lane >> 3][wid] = v;
     __syncthreads();
     if (wid == 0) {
-        const int nw = blockDim.x >> 5;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            double v = lane < nw ? red[c][lane] : 0.0;
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-            if (lane == 0 && A.partials) A.partials[blockIdx.x * 4 + c] = v;
-        }
+        double t = red[lane >> 3][lane & 7];
+        for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if ((lane & 7) == 0 && A.partials) A.partials[blockIdx.x * 4 + (lane >> 3)] = t;
     }
 }
 
@@ -1591,22 +1607,14 @@ __global__ void __launch_bounds__(256) noneq_kernel(const MomArgs<real> A)
     }
 }
 
-// Sum the per-block partials in a fixed order (one block): totals[4].
-static __global__ void __launch_bounds__(256) totals_kernel(const double *partials, int nblocks, double *totals)
+// Sum the per-block partials in a fixed order (one block, a warp per total).
+static __global__ void __launch_bounds__(128) totals_kernel(const double *partials, int nblocks, double *totals)
 {
-    __shared__ double red[4][256];
-    for (int c = 0; c < 4; ++c) {
-        double v = 0.0;
-        for (int b = threadIdx.x; b < nblocks; b += blockDim.x) v += partials[b * 4 + c];
-        red[c][threadIdx.x] = v;
-    }
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w)
-            for (int c = 0; c < 4; ++c) red[c][threadIdx.x] += red[c][threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x < 4) totals[threadIdx.x] = red[threadIdx.x][0];
+    const int c = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double v = 0.0;
+    for (int b = lane; b < nblocks; b += 32) v += partials[b * 4 + c];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) totals[c] = v;
 }
 
 }  // namespace dbm

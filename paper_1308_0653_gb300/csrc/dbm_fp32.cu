@@ -40,7 +40,7 @@ cudaError_t launch_row32(const StepArgs<float> &A, int steps, cudaStream_t s)
 
 cudaError_t launch_totals(const double *partials, int nblocks, double *totals, cudaStream_t s)
 {
-    totals_kernel<<<1, 256, 0, s>>>(partials, nblocks, totals);
+    totals_kernel<<<1, 128, 0, s>>>(partials, nblocks, totals);
     return cudaGetLastError();
 }
 

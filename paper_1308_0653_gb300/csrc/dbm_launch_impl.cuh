@@ -170,7 +170,7 @@ cudaError_t launch_init<DBM_REAL>(const InitArgs<DBM_REAL> &A, cudaStream_t s)
 template <>
 cudaError_t launch_moments<DBM_REAL>(const MomArgs<DBM_REAL> &A, int grid, cudaStream_t s)
 {
-    moments_kernel<DBM_REAL><<<grid, 256, 0, s>>>(A);
+    moments_kernel<DBM_REAL><<<grid, MOMENT_THREADS, 0, s>>>(A);
     return cudaGetLastError();
 }
 
