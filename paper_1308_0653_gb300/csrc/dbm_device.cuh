@@ -178,6 +178,20 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity
     return true;
 }
 
+// As mbar_try_wait, without suspending: only asks.
+__device__ __forceinline__ bool mbar_test_wait(uint64_t *bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(smem_addr(bar)), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
 __device__ __forceinline__ void mbar_arrive(uint64_t *bar)
 {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
@@ -1037,86 +1051,98 @@ __device__ __forceinline__ void march2(const Work &work, unsigned char *smem_raw
         if (lane == 0) issued_total = issued;
     } else {
         // ------------------------------ consumers -----------------------------
-        int base = 0;
         int parity = 0;
         bool ok = true;
-        // One work item: rows [mb, me) of the strip starting at radial site j0.
         real *stage = sm + NSTAGE * SLOT + warp * (NV * 32);  // STAGE: this warp's outgoing row
+        // Ring position taken next: slot and phase parity.  A wait, even for a row
+        // that has landed, takes some 150 cycles, so each row asks for the next
+        // one's barrier in the middle of its own arithmetic (`landed`).
+        int slot = 0;
+        uint32_t phase = 0;
+        bool landed = false;
+        auto ask = [&]() { landed = mbar_test_wait(&full[slot], phase); };
+        auto take = [&](const StepArgs<real> &A) -> int {
+            if (!landed) {
+                if (!mbar_wait_bounded(&full[slot], phase)) {
+                    if (lane == 0) atomicOr(A.status, ST_WAIT_TIMEOUT);
+                    abort_flag = 1;
+                }
+                if (*(volatile int *)&abort_flag) ok = false;
+            }
+            landed = false;
+            const int taken = slot;
+            if (++slot == NSTAGE) {
+                slot = 0;
+                phase ^= 1u;
+            }
+            return taken;
+        };
+        // One work item: rows [mb, me) of the strip starting at radial site j0.
         auto run_item = [&](const StepArgs<real> &A, const StepConsts<real> &C, const CUtensorMap *out_map, int j0,
                             int mb, int me) {
-            const int L = me - mb;
             const int j = j0 + tx;
             const bool active = j < A.nr;
             const real inv_r = A.inv_r[active ? j : 0];
-            for (int c = 1; c <= L; ++c) {
-                const int P = base + c;
-                for (int Q = (c == 1 ? P - 1 : P + 1); Q <= P + 1; ++Q) {
-                    if (!mbar_wait_bounded(&full[Q % NSTAGE], (uint32_t)((Q / NSTAGE) & 1))) {
-                        if (lane == 0) atomicOr(A.status, ST_WAIT_TIMEOUT);
-                        abort_flag = 1;
-                    }
-                }
-                if (*(volatile int *)&abort_flag) {
-                    ok = false;
-                    return;
-                }
-                const real *sc = sm + (P % NSTAGE) * SLOT;
+            int s_prev = take(A), s_cur = take(A);
+            for (int m = mb; m < me; ++m) {
+                const int s_next = take(A);
+                if (!ok) return;
+                real *sc = sm + s_cur * SLOT;
+                const real *sp = sm + s_prev * SLOT, *sn = sm + s_next * SLOT, *rt = sc + RTOFF;
+                const bool ghost = C.centre == 2 && j == 0;
                 if constexpr (sizeof(real) == 8) {  // every lane takes part (idle ones store nothing)
-                    const bool ghost = C.centre == 2 && j == 0;
-                    if (ghost)
-                        fill_centre_ghost<real, WP, LAMOFF, HALO>(A, sm + (P % NSTAGE) * SLOT, mb + c - 1);
+                    ask();
+                    if (ghost) fill_centre_ghost<real, WP, LAMOFF, HALO>(A, sc, m);
                     __syncwarp();
-                    site_update64_ring<WP, LAMOFF, HALO>(A, C, sm + ((P - 1) % NSTAGE) * SLOT, sc,
-                                                         sm + ((P + 1) % NSTAGE) * SLOT, j0, tx, mb + c - 1,
-                                                         sc + RTOFF);
+                    site_update64_ring<WP, LAMOFF, HALO>(A, C, sp, sc, sn, j0, tx, m, rt);
                     if (ghost) fence_proxy_async_smem();
+                    __syncwarp();
                 } else if (STAGE ? !Work::kCopyArgs || j - lane < A.nr : active) {
                     // STAGE: whole warps.  A batch, with many narrow last strips, leaves
                     // out warps without a site (1 % of its time; the test costs a single
                     // simulation 2 to 4 %).
                     real cs[4], sn4[4];
-                    const real *rt = sc + RTOFF;
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
                         cs[i] = rt[i];
                         sn4[i] = rt[8 + i];
                     }
-                    const bool ghost = C.centre == 2 && j == 0;
-                    if (ghost)
-                        fill_centre_ghost<real, WP, LAMOFF, HALO>(A, sm + (P % NSTAGE) * SLOT, mb + c - 1);
-                    const real *sp = sm + ((P - 1) % NSTAGE) * SLOT, *sn = sm + ((P + 1) % NSTAGE) * SLOT;
+                    if (ghost) fill_centre_ghost<real, WP, LAMOFF, HALO>(A, sc, m);
                     if constexpr (STAGE) {
-                        ring_site_update<WP, LAMOFF>(A, C, sp, sc, sn, HALO + tx, j, mb + c - 1, inv_r, cs, sn4, active,
-                                                [&](int q, float v) {
-                                                    if (q == 0) {  // the store before has read the staging row
-                                                        if (lane == 0) bulk_wait_read();
-                                                        __syncwarp();
-                                                    }
-                                                    stage[q * 32 + lane] = v;
-                                                });
+                        ring_site_update<WP, LAMOFF>(A, C, sp, sc, sn, HALO + tx, j, m, inv_r, cs, sn4, active,
+                                                     [&](int q, float v) {
+                                                         if (q == 0) {
+                                                             ask();
+                                                             // the store before has read the staging row
+                                                             if (lane == 0) bulk_wait_read();
+                                                             __syncwarp();
+                                                         }
+                                                         stage[q * 32 + lane] = v;
+                                                     });
                         fence_proxy_async_smem();
                         __syncwarp();
                         if (lane == 0 && (Work::kCopyArgs || j < A.nr)) {
-                            tma_store_3d(out_map, stage, j, mb + c - 1, 0);
+                            tma_store_3d(out_map, stage, j, m, 0);
                             bulk_commit();
                         }
                     } else {
-                        real *out = A.f_out + (long long)(mb + c - 1) * A.ld + j;
-                        ring_site_update<WP, LAMOFF>(A, C, sp, sc, sn, HALO + tx, j, mb + c - 1, inv_r, cs, sn4, true,
-                                                [&](int q, float v) { out[(long long)q * A.plane] = v; });
+                        real *out = A.f_out + (long long)m * A.ld + j;
+                        ring_site_update<WP, LAMOFF>(A, C, sp, sc, sn, HALO + tx, j, m, inv_r, cs, sn4, true,
+                                                     [&](int q, float v) { out[(long long)q * A.plane] = v; });
+                        if (ghost) fence_proxy_async_smem();
                     }
-                    if (ghost) fence_proxy_async_smem();
                 }
                 __syncwarp();
                 if (lane == 0) {
-                    mbar_arrive(&empty[(P - 1) % NSTAGE]);
-                    if (c == L) {
-                        mbar_arrive(&empty[P % NSTAGE]);
-                        mbar_arrive(&empty[(P + 1) % NSTAGE]);
+                    mbar_arrive(&empty[s_prev]);
+                    if (m == me - 1) {
+                        mbar_arrive(&empty[s_cur]);
+                        mbar_arrive(&empty[s_next]);
                     }
                 }
+                s_prev = s_cur;
+                s_cur = s_next;
             }
-            base += L + 2;
         };
         for (int it = blockIdx.x; it < nitems && ok; it += gridDim.x) {
             const StepArgs<real> *ga;
