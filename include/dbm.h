@@ -262,10 +262,10 @@ int dbm_import_state(dbm_t *h, const void *f, const void *lam, int64_t steps, vo
 
 /* Launch shape of the handle (any pointer may be NULL): persistent CTAs in
  * the grid, threads per CTA, dynamic shared memory per CTA, theta rows per
- * work item, work items per step and the step-kernel variant.  (FP64 variant 2
- * steps a single simulation by a kernel without work items, a warp per 32
- * radial sites of a row; its values are those of the row-ring kernel that a
- * batch runs for that variant.) */
+ * work item, work items per step and the step-kernel variant.  (FP64 variant 2,
+ * and FP32 variant 4 on small grids and single rows, step a simulation by
+ * kernels without work items; the values are then those of the row-ring kernel
+ * that a batch runs for that variant.) */
 int dbm_launch_info(const dbm_t *h, int *grid, int *threads, int *smem_bytes,
                     int *rows_per_item, int *items, int *variant);
 

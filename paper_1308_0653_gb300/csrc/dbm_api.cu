@@ -438,6 +438,44 @@ long long size_class(const dbm_params &p)
     return ((long long)p.precision << 16) | ((long long)lg(p.nr) << 8) | lg(p.ntheta);
 }
 
+// FP32 grids up to four waves of 16 warps per SM step straight from global memory.
+bool direct32_grid(const dbm_params &p, int nsm)
+{
+    return (long long)((p.nr + 31) / 32) * p.ntheta <= 64LL * nsm;
+}
+
+// Rows that the busiest CTA of an FP32 ring loads per step (0: not known).
+long long ring_rows(const dbm_params &p, int variant, int nsm)
+{
+    KernelInfo ki;
+    int32_t rows = 0;
+    int64_t items = 0;
+    if (kernel_info<float>(variant, &ki) != cudaSuccess || ki.blocks_per_sm < 1) return 0;
+    const long long slots = (long long)nsm * ki.blocks_per_sm;
+    if (dbm_plan_items(p.nr, p.ntheta, ki.W, (int32_t)slots, 0, &rows, &items) != DBM_OK) return 0;
+    return (items + slots - 1) / slots * (rows + 2);
+}
+
+// FP32 grids whose two states fit in L2: a step takes as long as its busiest CTA,
+// 1.75 us per row with two CTAs per SM and 2.35 with three (variant 5), so three
+// where the shorter items make up for that: its rows at most 11/15 of theirs
+// (777 x 501, 10 rows against 14, 23.1 -> 21.4 us per step, 512 x 768 20.7 -> 18.9;
+// at 9/12 600^2 19.4 against 19.0 but 1492 x 270 21.2 against 21.4).  Larger grids
+// wait for HBM, where it makes no difference (1024^2 49.1 against 49.8, 2048 x 512
+// 48.9 against 50.1).
+int pick_ring32(const dbm_params &p)
+{
+    const int two = default_variant<float>(), three = 5;
+    int dev = 0, nsm = 0, l2 = 0;
+    if (p.rows_per_item > 0 || p.ntheta == 1 || cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess || direct32_grid(p, nsm))
+        return two;
+    if (2LL * 33 * sizeof(float) * padded_ld(p.nr) * p.ntheta > l2) return two;
+    const long long r2 = ring_rows(p, two, nsm), r3 = ring_rows(p, three, nsm);
+    return r2 > 0 && r3 > 0 && 15 * r3 <= 11 * r2 ? three : two;
+}
+
 int pick_variant(const dbm_params &p)
 {
     if (p.variant > 0) return p.variant;
@@ -446,7 +484,7 @@ int pick_variant(const dbm_params &p)
         auto it = g_tuned.find(size_class(p));
         if (it != g_tuned.end()) return it->second;
     }
-    return p.precision == DBM_FP64 ? default_variant<double>() : default_variant<float>();
+    return p.precision == DBM_FP64 ? default_variant<double>() : pick_ring32(p);
 }
 
 // The FP64 direct kernel's tasks.  A warp task is 32 sites of a row; the SM
@@ -486,7 +524,7 @@ Path pick_path(const dbm_t *h)
         return h->variant == default_variant<double>() && warps <= (1 << 29) ? PATH_DIRECT64 : PATH_RING;
     if (h->variant != default_variant<float>()) return PATH_RING;
     if (p.ntheta == 1) return PATH_ROW32;
-    return warps <= 64LL * h->nsm ? PATH_DIRECT32 : PATH_RING;
+    return direct32_grid(p, h->nsm) ? PATH_DIRECT32 : PATH_RING;
 }
 
 // Launch shape for a kernel variant: persistent CTAs, one per resident slot,

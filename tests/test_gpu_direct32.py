@@ -73,3 +73,30 @@ def test_nan_in_lambda_reaches_f(nr, nth):
     bad = np.zeros((nth, nr), dtype=bool)
     bad[nth - 1, 33] = True
     assert np.isnan(f2[:, bad]).all() and np.isfinite(f2[:, ~bad]).all()
+
+
+@pytest.mark.parametrize("nr,nth,variant", [
+    (385, 880, 5), (1001, 311, 5), (777, 501, 5),         # items short enough, ragged last strips
+    (417, 800, 4), (600, 600, 4),                         # not short enough
+    (2048, 512, 4),                                       # two states beyond L2
+    (1000, 1, 4), (64, 64, 4),                            # the kernels without items
+])
+@pytest.mark.parametrize("shape", [{}, dict(sector=1, r_in=0.0, r_bc_inner="centre")])
+def test_shape_of_the_row_ring(nr, nth, variant, shape):
+    """Three CTAs per SM where the rule asks for them, with the other shapes' bits."""
+    from paper_1308_0653_gb300 import dbm
+    w = _workload(nr, nth, **shape)
+    got = []
+    for v in (0, 4, 5):
+        sim = dbm.Simulation(dict(w.params, precision="fp32", variant=v))
+        assert sim.launch_info()["variant"] == (v or variant)
+        sim.init_state(w.fields)
+        for n in (1, 33, 2):
+            sim.step(n)
+        f, lam, _ = sim.export_state()
+        assert dbm.dbm_status(sim.h) == dbm.DBM_OK
+        got.append((f, lam))
+        sim.close()
+    assert np.isfinite(got[0][0]).all()
+    for f, lam in got[1:]:
+        assert np.array_equal(f, got[0][0]) and np.array_equal(lam, got[0][1])
