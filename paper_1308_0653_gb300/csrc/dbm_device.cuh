@@ -1159,19 +1159,19 @@ __device__ __forceinline__ void march2(const Work &work, unsigned char *smem_raw
                 named_bar_sync(1, W);
                 parity ^= 1;
                 if (STAGE && lane == 0) fence_tensormap_acquire(&ga->tm_out);
-                // FP32: the item's pointers and sizes from there, and its
-                // constants from the batch constant table, into registers for
-                // the item (a single instance reads its constants from the
-                // constant bank as instruction operands).  The table is
-                // constant memory, so where registers run short the compiler
-                // can load a constant again instead of spilling it.  FP64 is
-                // bound by its arithmetic pipe and short of registers: it
-                // reads them where they are.
-                const StepConsts<real> &C = batch_consts<real>(cidx);
+                // FP32: the item's pointers and sizes from there into registers
+                // for the item.  Its constants stay in the batch constant
+                // table, at an index that the reduction makes uniform: they
+                // come through uniform registers, where copies of them took
+                // some 30 registers of every thread (24 instances of 128 to
+                // 640 sites squared 211 -> 206 us per step, 8 of 128 to 512
+                // 62 -> 59; a single instance reads its constants from the
+                // constant bank as instruction operands).  FP64 is bound by
+                // its arithmetic pipe.
+                const StepConsts<real> &C = batch_consts<real>((int)__reduce_or_sync(0xffffffffu, (unsigned)cidx));
                 if constexpr (sizeof(real) == 4) {
                     const StepArgs<real> Areg = *dst;
-                    const StepConsts<real> Creg = C;
-                    run_item(Areg, Creg, &ga->tm_out, j0, mb, me);
+                    run_item(Areg, C, &ga->tm_out, j0, mb, me);
                 } else {
                     run_item(*dst, C, &ga->tm_out, j0, mb, me);
                 }
