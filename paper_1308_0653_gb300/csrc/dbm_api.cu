@@ -495,8 +495,7 @@ void fill_direct64(dbm_t *h)
 {
     const dbm_params &p = h->p;
     const long long chunks = (p.nr + 31) / 32, tasks = chunks * p.ntheta, quarters = 4LL * h->nsm;
-    long long full = tasks / quarters * quarters;
-    if (4 * (tasks - full) > 2 * quarters) full = tasks;
+    const long long full = direct64_full(tasks, quarters);
     // Beside full tasks the few quarters left over share their SMs' FP64 pipe with
     // them: one or two to a block where that spreads them over more SMs (20000 x
     // 1: 68 quarters on 68 SMs instead of 17, 24.4 -> 20.4 us per step).
@@ -1320,6 +1319,7 @@ struct dbm_batch_s {
     int forced_variant;       // 0: the precision's default (set by dbm_batch_autotune)
     int grid;
     int nsm;
+    int blocks64;             // resident blocks per SM of the FP64 direct kernel
     cudaGraphExec_t graph;    // GRAPH_STEPS batch steps + counter advance
 };
 
@@ -1394,7 +1394,7 @@ BatchLayout batch_layout(int max_slots, long long max_items, int precision)
     L.items = off;
     off = align256(off + (size_t)max_items * sizeof(int4));
     L.nitems = off;
-    off = align256(off + sizeof(int));
+    off = align256(off + 2 * sizeof(int));
     L.T = off;
     off = align256(off + sizeof(long long));
     L.total = off;
@@ -1431,11 +1431,21 @@ void const_free(int device, int precision, int first, int n)
     for (int k = first; k < first + n && k < (int)used.size(); ++k) used[k] = 0;
 }
 
+// Units of a simulation stepped straight from global memory: warps' tasks of 32
+// sites (FP64); *chunks of them per row.
+int direct_units(const dbm_params &p, int *chunks)
+{
+    *chunks = (p.nr + 31) / 32;
+    return *chunks * p.ntheta;
+}
+
 template <typename real>
-void fill_slot(dbm_batch_t *b, int s, unsigned char *dst)
+void fill_slot(dbm_batch_t *b, int s, int &units, unsigned char *dst)
 {
     BatchSlot<real> sl;
     std::memset(&sl, 0, sizeof(sl));
+    sl.first = units;
+    if (b->inst[s]) units += direct_units(b->inst[s]->p, &sl.chunks);
     sl.cidx = b->cbase + s;
     StepConsts<real> *cst = reinterpret_cast<StepConsts<real> *>(b->cstage) + s;
     std::memset(cst, 0, sizeof(*cst));
@@ -1516,13 +1526,13 @@ int batch_launch(dbm_batch_t *b, int s, cudaStream_t st)
         BatchArgs<double> B{reinterpret_cast<const BatchSlot<double> *>(b->buf + b->off_slots),
                             reinterpret_cast<const int4 *>(b->buf + b->off_items),
                             reinterpret_cast<const int *>(b->buf + b->off_nitems),
-                            reinterpret_cast<const long long *>(b->buf + b->off_T), s};
-        e = launch_batch_step<double>(b->variant, B, b->grid, st);
+                            reinterpret_cast<const long long *>(b->buf + b->off_T), s, b->max_slots};
+        e = launch_batch_direct64(B, b->nsm, b->blocks64, st);
     } else {
         BatchArgs<float> B{reinterpret_cast<const BatchSlot<float> *>(b->buf + b->off_slots),
                            reinterpret_cast<const int4 *>(b->buf + b->off_items),
                            reinterpret_cast<const int *>(b->buf + b->off_nitems),
-                           reinterpret_cast<const long long *>(b->buf + b->off_T), s};
+                           reinterpret_cast<const long long *>(b->buf + b->off_T), s, b->max_slots};
         e = launch_batch_step<float>(b->variant, B, b->grid, st);
     }
     if (e != cudaSuccess) return cuda_fail(e, "batch step kernel launch");
@@ -1651,8 +1661,9 @@ int dbm_batch_create(int max_slots, int64_t max_items, int precision, int rows_p
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     b->variant = precision == DBM_FP64 ? default_variant<double>() : default_variant<float>();
     if (e == cudaSuccess)
-        e = precision == DBM_FP64 ? batch_kernel_info<double>(b->variant, &b->ki)
+        e = precision == DBM_FP64 ? kernel_info<double>(b->variant, &b->ki)
                                   : batch_kernel_info<float>(b->variant, &b->ki);
+    if (e == cudaSuccess) e = batch_direct64_blocks(&b->blocks64);
     if (e == cudaSuccess) e = cudaHostAlloc(&b->stage, L.items + (size_t)max_items * sizeof(int4) + 256,
                                             cudaHostAllocDefault);
     if (e == cudaSuccess) e = cudaHostAlloc(&b->cstage, (size_t)max_slots * sizeof(StepConsts<double>),
@@ -1742,13 +1753,13 @@ int dbm_batch_commit(dbm_batch_t *b, void *stream)
         int v = b->forced_variant > 0 ? b->forced_variant
                 : (b->precision == DBM_FP64 ? default_variant<double>() : default_variant<float>());
         KernelInfo ki;
-        CK(b->precision == DBM_FP64 ? batch_kernel_info<double>(v, &ki) : batch_kernel_info<float>(v, &ki));
+        CK(b->precision == DBM_FP64 ? kernel_info<double>(v, &ki) : batch_kernel_info<float>(v, &ki));
         bool maps_ok = true;
         for (int s = 0; s < b->max_slots; ++s)
             if (b->inst[s] && (!b->inst[s]->tmap_ok || b->inst[s]->ki.W != ki.W)) maps_ok = false;
         if (ki.version == 3 && !maps_ok) {
             v = b->precision == DBM_FP64 ? fallback_variant<double>() : fallback_variant<float>();
-            CK(b->precision == DBM_FP64 ? batch_kernel_info<double>(v, &ki) : batch_kernel_info<float>(v, &ki));
+            CK(b->precision == DBM_FP64 ? kernel_info<double>(v, &ki) : batch_kernel_info<float>(v, &ki));
         }
         if (v != b->variant) {
             if (b->graph) {  // captured with the other kernel
@@ -1771,12 +1782,13 @@ int dbm_batch_commit(dbm_batch_t *b, void *stream)
         b->stage_pending = false;
     }
     unsigned char *slots = b->stage;
+    int units = 0;  // of the slots so far, stepped straight from global memory
     int4 *items = reinterpret_cast<int4 *>(b->stage + b->off_items);
     for (int s = 0; s < b->max_slots; ++s) {
         if (b->precision == DBM_FP64)
-            fill_slot<double>(b, s, slots + (size_t)s * b->slot_bytes);
+            fill_slot<double>(b, s, units, slots + (size_t)s * b->slot_bytes);
         else
-            fill_slot<float>(b, s, slots + (size_t)s * b->slot_bytes);
+            fill_slot<float>(b, s, units, slots + (size_t)s * b->slot_bytes);
     }
     std::vector<int32_t> nr(b->max_slots, 0), nth(b->max_slots, 0), rows(b->max_slots, 0);
     for (int s = 0; s < b->max_slots; ++s) {
@@ -1791,7 +1803,8 @@ int dbm_batch_commit(dbm_batch_t *b, void *stream)
     if (rc != DBM_OK) return rc;
     n = planned;
     b->n_items = (int)n;
-    std::memcpy(b->stage + b->off_nitems, &b->n_items, sizeof(int));
+    const int words[2] = {b->n_items, units};
+    std::memcpy(b->stage + b->off_nitems, words, sizeof(words));
     CK(cudaMemcpyAsync(b->buf + b->off_slots, b->stage, (size_t)b->max_slots * b->slot_bytes,
                        cudaMemcpyHostToDevice, st));
     CK(b->precision == DBM_FP64
@@ -1802,7 +1815,7 @@ int dbm_batch_commit(dbm_batch_t *b, void *stream)
     if (n > 0)
         CK(cudaMemcpyAsync(b->buf + b->off_items, b->stage + b->off_items, (size_t)n * sizeof(int4),
                            cudaMemcpyHostToDevice, st));
-    CK(cudaMemcpyAsync(b->buf + b->off_nitems, b->stage + b->off_nitems, sizeof(int),
+    CK(cudaMemcpyAsync(b->buf + b->off_nitems, b->stage + b->off_nitems, sizeof(words),
                        cudaMemcpyHostToDevice, st));
     CK(cudaEventRecord(b->stage_ev, st));
     b->stage_pending = true;

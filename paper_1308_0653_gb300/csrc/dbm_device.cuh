@@ -668,15 +668,61 @@ struct BatchSlot {
     long long start, end;
     int par0;                // the instance's buffer index at global step start
     int cidx;                // the instance's entry in the batch constant table
+    int first, chunks;       // straight from global memory: units of the slots before, units per band of rows
 };
 
 template <typename real>
 struct BatchArgs {
     const BatchSlot<real> *slots;
     const int4 *items;        // (slot, j0, mb, me)
-    const int *n_items;       // device word: number of valid items
+    const int *n_items;       // device words: number of valid items, units of all slots
     const long long *T;       // device word: global step at the start of this replay
     int s;                    // step index within the replay
+    int max_slots;
+};
+
+// What a unit of a batch stepped straight from global memory needs of its slot.
+template <typename real>
+struct DirectSlot {
+    const real *f_in, *lam_in, *rowtab, *inv_r;
+    real *f_out, *lam_out;
+    int *status;
+    long long plane;
+    int nr, ntheta, ld;
+    int first, chunks;
+    int cidx;  // < 0: does not advance in this step
+};
+
+// Such a batch's slots, 32 at a time in shared memory, so that a unit's loads
+// do not wait for a chain of table look-ups; the lanes hold the first units.
+// An empty slot has no units: the last slot whose first is not beyond a unit
+// is the unit's.  Called by all threads of a block.
+template <typename real>
+struct DirectSlots {
+    int first;  // this lane's slot's
+    int end;    // the group's last unit + 1
+    int total;  // of all units
+    __device__ __forceinline__ void load(const BatchArgs<real> &B, int base, DirectSlot<real> (&slots)[32])
+    {
+        const int s = base + (threadIdx.x & 31);
+        total = B.n_items[1];
+        end = base + 32 < B.max_slots ? B.slots[base + 32].first : total;
+        first = s < B.max_slots ? B.slots[s].first : 0x7fffffff;
+        __syncthreads();  // the group before is done with
+        if (threadIdx.x < 32 && s < B.max_slots) {
+            const BatchSlot<real> &sl = B.slots[s];
+            const long long T = *B.T + B.s;
+            const StepArgs<real> &A = sl.args[(int)((T - sl.start + sl.par0) & 1)];
+            slots[threadIdx.x] = {A.f_in, A.lam_in, A.rowtab, A.inv_r, A.f_out, A.lam_out, A.status, A.plane, A.nr,
+                                  A.ntheta, A.ld, first, sl.chunks, T < sl.start || T >= sl.end ? -1 : sl.cidx};
+        }
+        __syncthreads();
+    }
+    // The slot of a unit of the group, by all lanes of a warp.
+    __device__ __forceinline__ int of(int unit) const
+    {
+        return __popc(__ballot_sync(0xffffffffu, first <= unit)) - 1;
+    }
 };
 
 template <typename real, int W>
@@ -1159,22 +1205,17 @@ __device__ __forceinline__ void march2(const Work &work, unsigned char *smem_raw
                 named_bar_sync(1, W);
                 parity ^= 1;
                 if (STAGE && lane == 0) fence_tensormap_acquire(&ga->tm_out);
-                // FP32: the item's pointers and sizes from there into registers
-                // for the item.  Its constants stay in the batch constant
-                // table, at an index that the reduction makes uniform: they
-                // come through uniform registers, where copies of them took
-                // some 30 registers of every thread (24 instances of 128 to
-                // 640 sites squared 211 -> 206 us per step, 8 of 128 to 512
-                // 62 -> 59; a single instance reads its constants from the
-                // constant bank as instruction operands).  FP64 is bound by
-                // its arithmetic pipe.
+                // The item's pointers and sizes from there into registers for
+                // the item.  Its constants stay in the batch constant table,
+                // at an index that the reduction makes uniform: they come
+                // through uniform registers, where copies of them took some
+                // 30 registers of every thread (24 instances of 128 to 640
+                // sites squared 211 -> 206 us per step, 8 of 128 to 512 62 ->
+                // 59; a single instance reads its constants from the constant
+                // bank as instruction operands).
                 const StepConsts<real> &C = batch_consts<real>((int)__reduce_or_sync(0xffffffffu, (unsigned)cidx));
-                if constexpr (sizeof(real) == 4) {
-                    const StepArgs<real> Areg = *dst;
-                    run_item(Areg, C, &ga->tm_out, j0, mb, me);
-                } else {
-                    run_item(*dst, C, &ga->tm_out, j0, mb, me);
-                }
+                const StepArgs<real> Areg = *dst;
+                run_item(Areg, C, &ga->tm_out, j0, mb, me);
             } else {
                 run_item(*ga, ga->c, &ga->tm_out, j0, mb, me);
             }

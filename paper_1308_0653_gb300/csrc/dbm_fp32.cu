@@ -11,6 +11,7 @@
     X(4, 3, 128, 5, true, 2) X(5, 3, 128, 4, false, 3)
 #define DBM_DEFAULT_VARIANT 4
 #define DBM_FALLBACK_VARIANT 2
+#define DBM_RING_BATCH 1
 #define DBM_BATCH_CONST_SLOTS DBM_BATCH_CONST_FP32  // batch constant table entries (160 B each)
 #include "dbm_launch_impl.cuh"
 

@@ -10,10 +10,22 @@
     X(4, 3, 64, 5, false, 2) X(5, 3, 64, 4, false, 3)
 #define DBM_DEFAULT_VARIANT 2
 #define DBM_FALLBACK_VARIANT 2
+#define DBM_RING_BATCH 0  // batches run the direct kernel
 #define DBM_BATCH_CONST_SLOTS DBM_BATCH_CONST_FP64  // batch constant table entries (304 B each)
 #include "dbm_launch_impl.cuh"
 
 namespace dbm {
+cudaError_t launch_batch_direct64(const BatchArgs<double> &B, int nsm, int blocks_per_sm, cudaStream_t s)
+{
+    batch_direct64_kernel<double><<<nsm * blocks_per_sm, 128, 0, s>>>(B, nsm);
+    return cudaGetLastError();
+}
+
+cudaError_t batch_direct64_blocks(int *blocks_per_sm)
+{
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, (void *)batch_direct64_kernel<double>, 128, 0);
+}
+
 cudaError_t launch_direct64(const Direct64Args &D, cudaStream_t s)
 {
     // up to two waves of warps, each has an SM quarter (nearly) to itself and

@@ -1,7 +1,8 @@
 // Instantiates the kernels of one precision; included once per precision
 // translation unit with DBM_REAL and the variant list DBM_VARIANTS(X) defined,
 // X(id, version, W, NSTAGE, STAGE, MIN_BLOCKS_PER_SM), DBM_DEFAULT_VARIANT and
-// DBM_FALLBACK_VARIANT (the default when tensor maps are unavailable).
+// DBM_FALLBACK_VARIANT (the default when tensor maps are unavailable) and
+// DBM_RING_BATCH (whether batches run the row ring).
 // version 1: CTA-wide row barrier; 2: producer warp, per-array bulk copies;
 // 3: producer warp, tensor-map TMA tiles.
 #include "dbm_launch.h"
@@ -40,17 +41,19 @@ struct Variant<1, W, NS, ST, MB> {
     static constexpr int kSmem =
         (int)(sizeof(DBM_REAL) * NS * NARR * (W + 2 * Halo<DBM_REAL>::value) + 8 * NS);
     static void *single() { return (void *)step_kernel<DBM_REAL, W, NS>; }
-    static void *batch() { return (void *)batch_step_kernel<DBM_REAL, W, NS>; }
     static cudaError_t run(const StepArgs<DBM_REAL> &A, int g, cudaStream_t s)
     {
         step_kernel<DBM_REAL, W, NS><<<g, kThreads, kSmem, s>>>(A);
         return cudaGetLastError();
     }
+#if DBM_RING_BATCH
+    static void *batch() { return (void *)batch_step_kernel<DBM_REAL, W, NS>; }
     static cudaError_t run_batch(const BatchArgs<DBM_REAL> &B, int g, cudaStream_t s)
     {
         batch_step_kernel<DBM_REAL, W, NS><<<g, kThreads, kSmem, s>>>(B);
         return cudaGetLastError();
     }
+#endif
 };
 
 template <int W, int NS, bool ST, int MB, bool TM>
@@ -58,17 +61,19 @@ struct VariantV2 {
     static constexpr int kThreads = W + 32;
     static constexpr int kSmem = smem_bytes_v2<DBM_REAL, W, NS, ST>();
     static void *single() { return (void *)step_kernel_v2<DBM_REAL, W, NS, ST, MB, TM>; }
-    static void *batch() { return (void *)batch_step_kernel_v2<DBM_REAL, W, NS, ST, MB, TM>; }
     static cudaError_t run(const StepArgs<DBM_REAL> &A, int g, cudaStream_t s)
     {
         step_kernel_v2<DBM_REAL, W, NS, ST, MB, TM><<<g, kThreads, kSmem, s>>>(A);
         return cudaGetLastError();
     }
+#if DBM_RING_BATCH
+    static void *batch() { return (void *)batch_step_kernel_v2<DBM_REAL, W, NS, ST, MB, TM>; }
     static cudaError_t run_batch(const BatchArgs<DBM_REAL> &B, int g, cudaStream_t s)
     {
         batch_step_kernel_v2<DBM_REAL, W, NS, ST, MB, TM><<<g, kThreads, kSmem, s>>>(B);
         return cudaGetLastError();
     }
+#endif
 };
 
 template <int W, int NS, bool ST, int MB>
@@ -122,23 +127,24 @@ cudaError_t kernel_info<DBM_REAL>(int variant, KernelInfo *out)
 }
 
 template <>
-cudaError_t batch_kernel_info<DBM_REAL>(int variant, KernelInfo *out)
+cudaError_t launch_step<DBM_REAL>(int variant, const StepArgs<DBM_REAL> &A, int grid, cudaStream_t s)
 {
     switch (variant) {
 #define X(id, ver, W, NS, ST, MB) \
-    case id: return info_of<Variant<ver, W, NS, ST, MB>>(Variant<ver, W, NS, ST, MB>::batch(), ver, W, NS, out);
+    case id: return Variant<ver, W, NS, ST, MB>::run(A, grid, s);
         DBM_VARIANTS(X)
 #undef X
     default: return cudaErrorInvalidValue;
     }
 }
 
+#if DBM_RING_BATCH
 template <>
-cudaError_t launch_step<DBM_REAL>(int variant, const StepArgs<DBM_REAL> &A, int grid, cudaStream_t s)
+cudaError_t batch_kernel_info<DBM_REAL>(int variant, KernelInfo *out)
 {
     switch (variant) {
 #define X(id, ver, W, NS, ST, MB) \
-    case id: return Variant<ver, W, NS, ST, MB>::run(A, grid, s);
+    case id: return info_of<Variant<ver, W, NS, ST, MB>>(Variant<ver, W, NS, ST, MB>::batch(), ver, W, NS, out);
         DBM_VARIANTS(X)
 #undef X
     default: return cudaErrorInvalidValue;
@@ -156,6 +162,7 @@ cudaError_t launch_batch_step<DBM_REAL>(int variant, const BatchArgs<DBM_REAL> &
     default: return cudaErrorInvalidValue;
     }
 }
+#endif
 
 template <>
 cudaError_t launch_init<DBM_REAL>(const InitArgs<DBM_REAL> &A, cudaStream_t s)
