@@ -264,8 +264,7 @@ int dbm_import_state(dbm_t *h, const void *f, const void *lam, int64_t steps, vo
  * the grid, threads per CTA, dynamic shared memory per CTA, theta rows per
  * work item, work items per step and the step-kernel variant.  (FP64 variant 2,
  * and FP32 variant 4 on small grids and single rows, step a simulation by
- * kernels without work items; the values are then those of the row-ring kernel
- * that a batch runs for that variant.) */
+ * kernels without work items; the values are then those of its row ring.) */
 int dbm_launch_info(const dbm_t *h, int *grid, int *threads, int *smem_bytes,
                     int *rows_per_item, int *items, int *variant);
 
@@ -429,7 +428,8 @@ int dbm_batch_step(dbm_batch_t *b, int64_t nsteps, void *stream);
 
 /* Autotuner of a batch: times the precision's default kernel and the
  * bulk-copy kernel, each with 16, 32, 64 and size-scaled (-1) theta rows per
- * work item, for twice `steps` batched steps each (after 32 untimed steps;
+ * work item (of the row ring, also where the batch is small enough to step
+ * without work items), for twice `steps` batched steps each (after 32 untimed steps;
  * the better of the two timings counts) with CUDA events on `stream`, and
  * keeps the fastest.  The trials advance every attached simulation
  * (8 x (32 + 2 steps) steps at most); attach them with enough steps left.  *variant and *rows_per_item receive the choice;
@@ -441,7 +441,9 @@ int dbm_batch_autotune(dbm_batch_t *b, int steps, void *stream, int *variant, in
                        float *ms_per_step);
 
 /* Launch shape: persistent grid, current number of work items, rows per item,
- * kernel variant (as of the last commit).  Null outputs are skipped. */
+ * kernel variant (as of the last commit).  FP64 batches and small FP32 batches
+ * of the default variant step by a kernel without work items; the values are
+ * then those of the row ring.  Null outputs are skipped. */
 int dbm_batch_launch_info(const dbm_batch_t *b, int *grid, int *items, int *rows_per_item,
                           int *variant);
 

@@ -1319,8 +1319,10 @@ struct dbm_batch_s {
     int forced_variant;       // 0: the precision's default (set by dbm_batch_autotune)
     int grid;
     int nsm;
+    bool direct;              // FP32: steps straight from global memory (as of the last commit)
+    bool ring_only;           // while dbm_batch_autotune compares shapes of the row ring
     int blocks64;             // resident blocks per SM of the FP64 direct kernel
-    cudaGraphExec_t graph;    // GRAPH_STEPS batch steps + counter advance
+    cudaGraphExec_t graphs[2];  // GRAPH_STEPS batch steps + counter advance: row ring, direct
 };
 
 namespace {
@@ -1431,12 +1433,14 @@ void const_free(int device, int precision, int first, int n)
     for (int k = first; k < first + n && k < (int)used.size(); ++k) used[k] = 0;
 }
 
-// Units of a simulation stepped straight from global memory: warps' tasks of 32
-// sites (FP64); *chunks of them per row.
+// Units of a simulation stepped straight from global memory: tiles of 128 sites
+// (FP32), warps' tasks of 32 (FP64); *chunks of them per band of rows.
 int direct_units(const dbm_params &p, int *chunks)
 {
-    *chunks = (p.nr + 31) / 32;
-    return *chunks * p.ntheta;
+    const int log_cols = p.precision == DBM_FP64 ? 5 : direct32_log_cols(p.ntheta);
+    const int rows = p.precision == DBM_FP64 ? 1 : 128 >> log_cols;
+    *chunks = (p.nr + (1 << log_cols) - 1) >> log_cols;
+    return *chunks * ((p.ntheta + rows - 1) / rows);
 }
 
 template <typename real>
@@ -1519,6 +1523,16 @@ std::vector<PlanItem> balance_items(const std::vector<PlanItem> &items, int grid
     return out;
 }
 
+// An FP32 batch steps straight from global memory up to 16 tiles per SM, the line
+// of a single simulation's direct kernel: 16 instances of 64 to 160 sites squared
+// 18.8 -> 14.9 us per step, one of 64^2 5.2 -> 3.6, 2444 tiles 21.3 -> 20.7, but
+// 3113 tiles of two larger ones 25.1 -> 28.4.
+bool batch_direct32(const dbm_batch_t *b, int tiles)
+{
+    return b->precision == DBM_FP32 && !b->ring_only && b->variant == default_variant<float>() &&
+           tiles <= 16 * b->nsm;
+}
+
 int batch_launch(dbm_batch_t *b, int s, cudaStream_t st)
 {
     cudaError_t e;
@@ -1533,7 +1547,8 @@ int batch_launch(dbm_batch_t *b, int s, cudaStream_t st)
                            reinterpret_cast<const int4 *>(b->buf + b->off_items),
                            reinterpret_cast<const int *>(b->buf + b->off_nitems),
                            reinterpret_cast<const long long *>(b->buf + b->off_T), s, b->max_slots};
-        e = launch_batch_step<float>(b->variant, B, b->grid, st);
+        e = b->direct ? launch_batch_direct32(B, b->nsm, st)
+                      : launch_batch_step<float>(b->variant, B, b->grid, st);
     }
     if (e != cudaSuccess) return cuda_fail(e, "batch step kernel launch");
     return DBM_OK;
@@ -1558,12 +1573,12 @@ int batch_build_graph(dbm_batch_t *b)
         if (rc == DBM_OK) rc = batch_advance(b, GRAPH_STEPS, cs);
         e = cudaStreamEndCapture(cs, &g);
     }
-    if (e == cudaSuccess && rc == DBM_OK) e = cudaGraphInstantiate(&b->graph, g, 0);
+    if (e == cudaSuccess && rc == DBM_OK) e = cudaGraphInstantiate(&b->graphs[b->direct], g, 0);
     if (g) cudaGraphDestroy(g);
     cudaStreamDestroy(cs);
     if (rc != DBM_OK) return rc;
     if (e != cudaSuccess) {
-        b->graph = nullptr;
+        b->graphs[b->direct] = nullptr;
         return cuda_fail(e, "batch graph capture");
     }
     return DBM_OK;
@@ -1701,7 +1716,8 @@ int dbm_batch_destroy(dbm_batch_t *b)
     if (!b) return DBM_EINVAL;
     if (b->stage_pending) cudaEventSynchronize(b->stage_ev);
     cudaEventSynchronize(b->done);  // queued batched steps read the tables
-    if (b->graph) cudaGraphExecDestroy(b->graph);
+    for (cudaGraphExec_t g : b->graphs)
+        if (g) cudaGraphExecDestroy(g);
     cudaEventDestroy(b->stage_ev);
     cudaEventDestroy(b->done);
     cudaFreeHost(b->stage);
@@ -1762,10 +1778,10 @@ int dbm_batch_commit(dbm_batch_t *b, void *stream)
             CK(b->precision == DBM_FP64 ? kernel_info<double>(v, &ki) : batch_kernel_info<float>(v, &ki));
         }
         if (v != b->variant) {
-            if (b->graph) {  // captured with the other kernel
+            if (b->graphs[0]) {  // captured with the other kernel
                 CK(cudaStreamSynchronize(st));
-                cudaGraphExecDestroy(b->graph);
-                b->graph = nullptr;
+                cudaGraphExecDestroy(b->graphs[0]);
+                b->graphs[0] = nullptr;
             }
             b->variant = v;
             b->ki = ki;
@@ -1790,6 +1806,7 @@ int dbm_batch_commit(dbm_batch_t *b, void *stream)
         else
             fill_slot<float>(b, s, units, slots + (size_t)s * b->slot_bytes);
     }
+    b->direct = batch_direct32(b, units);
     std::vector<int32_t> nr(b->max_slots, 0), nth(b->max_slots, 0), rows(b->max_slots, 0);
     for (int s = 0; s < b->max_slots; ++s) {
         if (!b->inst[s]) continue;
@@ -1836,11 +1853,11 @@ int dbm_batch_step(dbm_batch_t *b, int64_t nsteps, void *stream)
     while (nsteps > 0) {
         int rc;
         if (nsteps >= GRAPH_STEPS) {
-            if (!b->graph) {
+            if (!b->graphs[b->direct]) {
                 rc = batch_build_graph(b);
                 if (rc != DBM_OK) return rc;
             }
-            CK(cudaGraphLaunch(b->graph, st));
+            CK(cudaGraphLaunch(b->graphs[b->direct], st));
             nsteps -= GRAPH_STEPS;
             b->T += GRAPH_STEPS;
         } else {
@@ -1878,6 +1895,7 @@ int dbm_batch_autotune(dbm_batch_t *b, int steps, void *stream, int *variant, in
     CK(cudaEventCreate(&e1));
     int rc = DBM_OK, bestv = 0, bestr = 0;
     float bestms = 0.f;
+    b->ring_only = true;
     for (int c = 0; c < 8 && rc == DBM_OK; ++c) {
         const int v = vs[c / 4], r = rows[c % 4];
         if (ms_per_step) ms_per_step[c] = 0.f;
@@ -1912,6 +1930,7 @@ int dbm_batch_autotune(dbm_batch_t *b, int steps, void *stream, int *variant, in
             bestms = ms;
         }
     }
+    b->ring_only = false;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (rc != DBM_OK) return rc;

@@ -18,7 +18,7 @@
 namespace dbm {
 cudaError_t launch_direct32(const StepArgs<float> &A, int nsm, cudaStream_t s)
 {
-    const int log_cols = A.ntheta >= 4 ? 5 : 7, cols = 1 << log_cols, rows = 128 >> log_cols;
+    const int log_cols = direct32_log_cols(A.ntheta), cols = 1 << log_cols, rows = 128 >> log_cols;
     const long long blocks = (long long)((A.nr + cols - 1) / cols) * ((A.ntheta + rows - 1) / rows);
     // Three blocks per SM (168 registers) or four (128): a block's time is 0.81
     // of that with four (64^2, one wave: 2.89 against 3.55 us per step), so what
@@ -30,6 +30,12 @@ cudaError_t launch_direct32(const StepArgs<float> &A, int nsm, cudaStream_t s)
         direct32_kernel<false, 3><<<(unsigned)blocks, 128, 0, s>>>(A, log_cols);
     else
         direct32_kernel<false, 4><<<(unsigned)blocks, 128, 0, s>>>(A, log_cols);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_batch_direct32(const BatchArgs<float> &B, int nsm, cudaStream_t s)
+{
+    batch_direct32_kernel<float><<<3 * nsm, 128, 0, s>>>(B);
     return cudaGetLastError();
 }
 

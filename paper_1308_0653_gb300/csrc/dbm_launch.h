@@ -40,6 +40,7 @@ template <typename real> cudaError_t batch_kernel_info(int variant, KernelInfo *
 template <typename real>
 cudaError_t launch_batch_step(int variant, const BatchArgs<real> &B, int grid, cudaStream_t s);
 // A batch's step straight from global memory.
+cudaError_t launch_batch_direct32(const BatchArgs<float> &B, int nsm, cudaStream_t s);
 cudaError_t launch_batch_direct64(const BatchArgs<double> &B, int nsm, int blocks_per_sm, cudaStream_t s);
 cudaError_t batch_direct64_blocks(int *blocks_per_sm);
 cudaError_t launch_batch_advance(long long *T, int k, cudaStream_t s);

@@ -1,6 +1,7 @@
-"""Batches stepped straight from global memory (every FP64 batch): uneven and
-tiny simulations, sectors, disc centres, empty slots, more than one group of 32
-slots and simulations that end at different steps, bit for bit against each
+"""Batches stepped straight from global memory (every FP64 batch, FP32 ones up to
+16 tiles per SM): uneven and tiny simulations, sectors, disc centres, empty slots,
+more than one group of 32 slots, simulations that end at different steps, and
+FP32 batches that cross the line between the kernels, bit for bit against each
 simulation alone in the row ring."""
 import numpy as np
 import pytest
@@ -52,7 +53,7 @@ SMALL = [(1, 8), (31, 3), (33, 5), (64, 4), (97, 1)]
 TURNED = [(40, 2, 1), (70, 9, 1, True), (60, 16, 0, True)]
 
 
-@pytest.mark.parametrize("precision", ["fp64"])
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
 @pytest.mark.parametrize("slots,shapes", [
     (1, [(33, 7)]),
     (8, SMALL + TURNED),
@@ -77,3 +78,23 @@ def test_same_bits_as_alone(slots, shapes, precision):
     for s, _, _ in sims:
         s.close()
 
+
+def test_across_the_line_between_the_kernels():
+    from paper_1308_0653_gb300 import dbm
+    b = dbm.Batch(4, 8192, precision="fp32")
+    ws = [_workload(96, 80), _workload(640, 620), _workload(130, 70)]
+    sims = []
+    for w in ws:
+        sims.append(dbm.Simulation(dict(w.params, precision="fp32")))
+        sims[-1].init_state(w.fields)
+    b.attach(0, sims[0], 1000)
+    b.step(34)             # straight from global memory
+    b.attach(1, sims[1], 1000)
+    b.step(34)             # the row ring
+    b.detach(1)
+    b.attach(3, sims[2], 1000)
+    b.step(35)
+    _check([(sims[0], ws[0], 103), (sims[1], ws[1], 34), (sims[2], ws[2], 35)], "fp32")
+    b.close()
+    for s in sims:
+        s.close()
