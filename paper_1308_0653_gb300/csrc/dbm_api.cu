@@ -514,7 +514,7 @@ void fill_direct64(dbm_t *h)
 // to four waves of 16 warps per SM: there the step is latency, and the ring takes
 // time to fill (64^2 4.1 -> 2.8 us per step, 256^2 6.5 -> 5.3, 512^2, the last
 // size below the line, 14.4 -> 13.6); beyond it the ring's long row copies win
-// (600^2 22.1 against 19.8, 2048^2 238 against 181).
+// (600^2 22.1 against 19.2, 2048^2 238 against 181).
 Path pick_path(const dbm_t *h)
 {
     const dbm_params &p = h->p;
@@ -1358,6 +1358,10 @@ int dbm_autotune(dbm_t *h, int steps, void *stream, int *best, float *ms_per_ste
 // ===========================================================================
 // Batches: many uneven instances advanced by one persistent launch per step.
 // ===========================================================================
+// How an FP32 batch steps: the row ring, its constants in registers or through
+// uniform ones, or straight from global memory.
+enum BatchPath { BATCH_RING, BATCH_RING_UNIFORM, BATCH_DIRECT, BATCH_PATHS };
+
 struct dbm_batch_s {
     int precision;
     int max_slots;
@@ -1385,10 +1389,10 @@ struct dbm_batch_s {
     int forced_variant;       // 0: the precision's default (set by dbm_batch_autotune)
     int grid;
     int nsm;
-    bool direct;              // FP32: steps straight from global memory (as of the last commit)
+    BatchPath path;           // FP32: how it steps (as of the last commit)
     bool ring_only;           // while dbm_batch_autotune compares shapes of the row ring
     int blocks64;             // resident blocks per SM of the FP64 direct kernel
-    cudaGraphExec_t graphs[2];  // GRAPH_STEPS batch steps + counter advance: row ring, direct
+    cudaGraphExec_t graphs[BATCH_PATHS];  // GRAPH_STEPS batch steps + counter advance
 };
 
 namespace {
@@ -1599,6 +1603,19 @@ bool batch_direct32(const dbm_batch_t *b, int tiles)
            tiles <= 16 * b->nsm;
 }
 
+// The row ring's way to a slot's constants.  Through uniform registers up to 40 000
+// sites per SM (24 instances of 128 to 640 sites squared 234 -> 230 us per step, 64
+// of 128 to 400 273 -> 269, 8 of 128 to 512 60 -> 57.6); larger batches wait for
+// HBM, where copies in every thread's registers are faster (48 of 128 to 640 417
+// against 427, 64 of 128 to 1024 1151 against 1252).
+bool batch_uniform(const dbm_batch_t *b)
+{
+    long long sites = 0;
+    for (const dbm_t *h : b->inst)
+        if (h) sites += (long long)h->p.nr * h->p.ntheta;
+    return sites <= 40000LL * b->nsm;
+}
+
 int batch_launch(dbm_batch_t *b, int s, cudaStream_t st)
 {
     cudaError_t e;
@@ -1613,8 +1630,8 @@ int batch_launch(dbm_batch_t *b, int s, cudaStream_t st)
                            reinterpret_cast<const int4 *>(b->buf + b->off_items),
                            reinterpret_cast<const int *>(b->buf + b->off_nitems),
                            reinterpret_cast<const long long *>(b->buf + b->off_T), s, b->max_slots};
-        e = b->direct ? launch_batch_direct32(B, b->nsm, st)
-                      : launch_batch_step<float>(b->variant, B, b->grid, st);
+        e = b->path == BATCH_DIRECT ? launch_batch_direct32(B, b->nsm, st)
+                                    : launch_batch_step<float>(b->variant, B, b->grid, b->path == BATCH_RING_UNIFORM, st);
     }
     if (e != cudaSuccess) return cuda_fail(e, "batch step kernel launch");
     return DBM_OK;
@@ -1639,12 +1656,12 @@ int batch_build_graph(dbm_batch_t *b)
         if (rc == DBM_OK) rc = batch_advance(b, GRAPH_STEPS, cs);
         e = cudaStreamEndCapture(cs, &g);
     }
-    if (e == cudaSuccess && rc == DBM_OK) e = cudaGraphInstantiate(&b->graphs[b->direct], g, 0);
+    if (e == cudaSuccess && rc == DBM_OK) e = cudaGraphInstantiate(&b->graphs[b->path], g, 0);
     if (g) cudaGraphDestroy(g);
     cudaStreamDestroy(cs);
     if (rc != DBM_OK) return rc;
     if (e != cudaSuccess) {
-        b->graphs[b->direct] = nullptr;
+        b->graphs[b->path] = nullptr;
         return cuda_fail(e, "batch graph capture");
     }
     return DBM_OK;
@@ -1844,11 +1861,12 @@ int dbm_batch_commit(dbm_batch_t *b, void *stream)
             CK(b->precision == DBM_FP64 ? kernel_info<double>(v, &ki) : batch_kernel_info<float>(v, &ki));
         }
         if (v != b->variant) {
-            if (b->graphs[0]) {  // captured with the other kernel
-                CK(cudaStreamSynchronize(st));
-                cudaGraphExecDestroy(b->graphs[0]);
-                b->graphs[0] = nullptr;
-            }
+            for (BatchPath r : {BATCH_RING, BATCH_RING_UNIFORM})
+                if (b->graphs[r]) {  // captured with the other kernel
+                    CK(cudaStreamSynchronize(st));
+                    cudaGraphExecDestroy(b->graphs[r]);
+                    b->graphs[r] = nullptr;
+                }
             b->variant = v;
             b->ki = ki;
             b->grid = b->nsm * std::max(1, ki.blocks_per_sm);
@@ -1872,7 +1890,7 @@ int dbm_batch_commit(dbm_batch_t *b, void *stream)
         else
             fill_slot<float>(b, s, units, slots + (size_t)s * b->slot_bytes);
     }
-    b->direct = batch_direct32(b, units);
+    b->path = batch_direct32(b, units) ? BATCH_DIRECT : batch_uniform(b) ? BATCH_RING_UNIFORM : BATCH_RING;
     std::vector<int32_t> nr(b->max_slots, 0), nth(b->max_slots, 0), rows(b->max_slots, 0);
     for (int s = 0; s < b->max_slots; ++s) {
         if (!b->inst[s]) continue;
@@ -1919,11 +1937,11 @@ int dbm_batch_step(dbm_batch_t *b, int64_t nsteps, void *stream)
     while (nsteps > 0) {
         int rc;
         if (nsteps >= GRAPH_STEPS) {
-            if (!b->graphs[b->direct]) {
+            if (!b->graphs[b->path]) {
                 rc = batch_build_graph(b);
                 if (rc != DBM_OK) return rc;
             }
-            CK(cudaGraphLaunch(b->graphs[b->direct], st));
+            CK(cudaGraphLaunch(b->graphs[b->path], st));
             nsteps -= GRAPH_STEPS;
             b->T += GRAPH_STEPS;
         } else {

@@ -725,9 +725,10 @@ struct DirectSlots {
     }
 };
 
-template <typename real, int W>
+// UNIFORM: a slot's constants through uniform registers (see march2).
+template <typename real, int W, bool UNIFORM = false>
 struct BatchWork {
-    static constexpr bool kCopyArgs = true;
+    static constexpr bool kCopyArgs = true, kUniform = UNIFORM;
     const BatchSlot<real> *slots;
     const int4 *items;
     int n;
@@ -1206,16 +1207,21 @@ __device__ __forceinline__ void march2(const Work &work, unsigned char *smem_raw
                 parity ^= 1;
                 if (STAGE && lane == 0) fence_tensormap_acquire(&ga->tm_out);
                 // The item's pointers and sizes from there into registers for
-                // the item.  Its constants stay in the batch constant table,
-                // at an index that the reduction makes uniform: they come
-                // through uniform registers, where copies of them took some
-                // 30 registers of every thread (24 instances of 128 to 640
-                // sites squared 211 -> 206 us per step, 8 of 128 to 512 62 ->
-                // 59; a single instance reads its constants from the constant
-                // bank as instruction operands).
-                const StepConsts<real> &C = batch_consts<real>((int)__reduce_or_sync(0xffffffffu, (unsigned)cidx));
+                // the item (a single instance reads its constants from the
+                // constant bank as instruction operands).  Its constants stay
+                // in the batch constant table, at an index that the reduction
+                // makes uniform, so that they come through uniform registers,
+                // or are copied into some 30 registers of every thread: which
+                // of the two is faster depends on the batch's size (see
+                // batch_uniform).
                 const StepArgs<real> Areg = *dst;
-                run_item(Areg, C, &ga->tm_out, j0, mb, me);
+                if constexpr (Work::kUniform) {
+                    run_item(Areg, batch_consts<real>((int)__reduce_or_sync(0xffffffffu, (unsigned)cidx)), &ga->tm_out, j0,
+                             mb, me);
+                } else {
+                    const StepConsts<real> Creg = batch_consts<real>(cidx);
+                    run_item(Areg, Creg, &ga->tm_out, j0, mb, me);
+                }
             } else {
                 run_item(*ga, ga->c, &ga->tm_out, j0, mb, me);
             }
@@ -1239,12 +1245,12 @@ __global__ void __launch_bounds__(W + 32, MINB) step_kernel_v2(const __grid_cons
     march2<real, W, NSTAGE, STAGE, TMAP>(work, smem_raw, nullptr);
 }
 
-template <typename real, int W, int NSTAGE, bool STAGE, int MINB, bool TMAP>
+template <typename real, int W, int NSTAGE, bool STAGE, int MINB, bool TMAP, bool UNIFORM>
 __global__ void __launch_bounds__(W + 32, MINB) batch_step_kernel_v2(const __grid_constant__ BatchArgs<real> B)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ __align__(64) StepArgs<real> sargs2[2];
-    BatchWork<real, W> work{B.slots, B.items, *B.n_items, *B.T + B.s};
+    BatchWork<real, W, UNIFORM> work{B.slots, B.items, *B.n_items, *B.T + B.s};
     march2<real, W, NSTAGE, STAGE, TMAP>(work, smem_raw, sargs2);
 }
 

@@ -38,7 +38,7 @@ cudaError_t launch_row32(const StepArgs<float> &A, int steps, cudaStream_t s);
 cudaError_t launch_direct64(const Direct64Args &D, cudaStream_t s);
 template <typename real> cudaError_t batch_kernel_info(int variant, KernelInfo *out);
 template <typename real>
-cudaError_t launch_batch_step(int variant, const BatchArgs<real> &B, int grid, cudaStream_t s);
+cudaError_t launch_batch_step(int variant, const BatchArgs<real> &B, int grid, bool uniform, cudaStream_t s);
 // A batch's step straight from global memory.
 cudaError_t launch_batch_direct32(const BatchArgs<float> &B, int nsm, cudaStream_t s);
 cudaError_t launch_batch_direct64(const BatchArgs<double> &B, int nsm, int blocks_per_sm, cudaStream_t s);

@@ -47,8 +47,8 @@ struct Variant<1, W, NS, ST, MB> {
         return cudaGetLastError();
     }
 #if DBM_RING_BATCH
-    static void *batch() { return (void *)batch_step_kernel<DBM_REAL, W, NS>; }
-    static cudaError_t run_batch(const BatchArgs<DBM_REAL> &B, int g, cudaStream_t s)
+    static void *batch(bool) { return (void *)batch_step_kernel<DBM_REAL, W, NS>; }
+    static cudaError_t run_batch(const BatchArgs<DBM_REAL> &B, int g, bool, cudaStream_t s)
     {
         batch_step_kernel<DBM_REAL, W, NS><<<g, kThreads, kSmem, s>>>(B);
         return cudaGetLastError();
@@ -67,10 +67,18 @@ struct VariantV2 {
         return cudaGetLastError();
     }
 #if DBM_RING_BATCH
-    static void *batch() { return (void *)batch_step_kernel_v2<DBM_REAL, W, NS, ST, MB, TM>; }
-    static cudaError_t run_batch(const BatchArgs<DBM_REAL> &B, int g, cudaStream_t s)
+    // the default (staged) variant has both ways to a slot's constants
+    static void *batch(bool uniform)
     {
-        batch_step_kernel_v2<DBM_REAL, W, NS, ST, MB, TM><<<g, kThreads, kSmem, s>>>(B);
+        return uniform && ST ? (void *)batch_step_kernel_v2<DBM_REAL, W, NS, ST, MB, TM, ST>
+                             : (void *)batch_step_kernel_v2<DBM_REAL, W, NS, ST, MB, TM, false>;
+    }
+    static cudaError_t run_batch(const BatchArgs<DBM_REAL> &B, int g, bool uniform, cudaStream_t s)
+    {
+        if (uniform && ST)
+            batch_step_kernel_v2<DBM_REAL, W, NS, ST, MB, TM, ST><<<g, kThreads, kSmem, s>>>(B);
+        else
+            batch_step_kernel_v2<DBM_REAL, W, NS, ST, MB, TM, false><<<g, kThreads, kSmem, s>>>(B);
         return cudaGetLastError();
     }
 #endif
@@ -144,7 +152,11 @@ cudaError_t batch_kernel_info<DBM_REAL>(int variant, KernelInfo *out)
 {
     switch (variant) {
 #define X(id, ver, W, NS, ST, MB) \
-    case id: return info_of<Variant<ver, W, NS, ST, MB>>(Variant<ver, W, NS, ST, MB>::batch(), ver, W, NS, out);
+    case id: { \
+        using V = Variant<ver, W, NS, ST, MB>; \
+        const cudaError_t e = info_of<V>(V::batch(true), ver, W, NS, out); \
+        return e != cudaSuccess ? e : info_of<V>(V::batch(false), ver, W, NS, out); \
+    }
         DBM_VARIANTS(X)
 #undef X
     default: return cudaErrorInvalidValue;
@@ -152,11 +164,11 @@ cudaError_t batch_kernel_info<DBM_REAL>(int variant, KernelInfo *out)
 }
 
 template <>
-cudaError_t launch_batch_step<DBM_REAL>(int variant, const BatchArgs<DBM_REAL> &B, int grid, cudaStream_t s)
+cudaError_t launch_batch_step<DBM_REAL>(int variant, const BatchArgs<DBM_REAL> &B, int grid, bool uniform, cudaStream_t s)
 {
     switch (variant) {
 #define X(id, ver, W, NS, ST, MB) \
-    case id: return Variant<ver, W, NS, ST, MB>::run_batch(B, grid, s);
+    case id: return Variant<ver, W, NS, ST, MB>::run_batch(B, grid, uniform, s);
         DBM_VARIANTS(X)
 #undef X
     default: return cudaErrorInvalidValue;

@@ -98,3 +98,25 @@ def test_across_the_line_between_the_kernels():
     b.close()
     for s in sims:
         s.close()
+
+
+def test_constants_either_way():
+    """The row ring's constants from registers (large batches) and through uniform registers."""
+    from paper_1308_0653_gb300 import dbm
+    b = dbm.Batch(3, 1 << 15, precision="fp32")
+    ws = [_workload(700, 600, v_scale=1.01), _workload(130, 70, sector=1), _workload(2500, 2450)]
+    sims = []
+    for w in ws:
+        sims.append(dbm.Simulation(dict(w.params, precision="fp32")))
+        sims[-1].init_state(w.fields)
+    b.attach(0, sims[0], 1000)
+    b.attach(1, sims[1], 1000)
+    b.step(34)             # 2800 sites per SM
+    b.attach(2, sims[2], 1000)
+    b.step(34)             # 43 000
+    b.detach(2)
+    b.step(35)
+    _check([(sims[0], ws[0], 103), (sims[1], ws[1], 103), (sims[2], ws[2], 34)], "fp32")
+    b.close()
+    for s in sims:
+        s.close()
