@@ -820,66 +820,14 @@ int dbm_destroy(dbm_t *h)
 
 }  // extern "C"
 
-// Blocks per SM of the init and moments kernels on pinned host arrays: enough to
-// keep the host link busy (about 205 GB/s to the device, 190 back, as the copy
-// engines), and room on the SMs for other streams.  Against copies in chunks
-// through device memory init and moments of 256^2 69 and 78 -> 61 and 59 us,
-// of 1024^2 297 and 324 -> 248 and 279 (the link alone takes 203 and 220).
-constexpr int HOST_BLOCKS = 1;
-constexpr int INIT_BLOCKS = 4096;
-
-// Five fields of N values each (any may be null where the caller allows it).
-struct Fields5 {
-    double *at[5];
-};
-
-static Fields5 planes(const double *base, size_t N)
-{
-    double *p = const_cast<double *>(base);
-    return {{p, p + N, p + 2 * N, p + 3 * N, p + 4 * N}};
-}
-
-// The device's addresses of host arrays of N doubles, where all of them are
-// pinned: each inside one allocation, aligned, apart from the others.
-static bool pinned_fields(const double *const (&host)[5], size_t N, Fields5 *dev)
-{
-    static const PFN_cuPointerGetAttribute_v4000 get = [] {
-        void *fn = nullptr;
-        cudaDriverEntryPointQueryResult found;
-        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &fn, 4000, cudaEnableDefault, &found) != cudaSuccess ||
-            found != cudaDriverEntryPointSuccess)
-            fn = nullptr;
-        return reinterpret_cast<PFN_cuPointerGetAttribute_v4000>(fn);
-    }();
-    if (!get) return false;
-    for (int k = 0; k < 5; ++k) {
-        dev->at[k] = nullptr;
-        if (!host[k]) continue;
-        const CUdeviceptr p = (CUdeviceptr)(uintptr_t)host[k];
-        unsigned type = 0;
-        CUdeviceptr start = 0, on_device = 0;
-        size_t size = 0;
-        if ((p & 7) || get(&type, CU_POINTER_ATTRIBUTE_MEMORY_TYPE, p) != CUDA_SUCCESS || type != CU_MEMORYTYPE_HOST ||
-            get(&start, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, p) != CUDA_SUCCESS ||
-            get(&size, CU_POINTER_ATTRIBUTE_RANGE_SIZE, p) != CUDA_SUCCESS || p < start ||
-            p - start + N * sizeof(double) > size ||
-            get(&on_device, CU_POINTER_ATTRIBUTE_DEVICE_POINTER, p) != CUDA_SUCCESS || !on_device || (on_device & 7))
-            return false;
-        dev->at[k] = reinterpret_cast<double *>((uintptr_t)on_device);
-        for (int i = 0; i < k; ++i)
-            if (dev->at[i] && dev->at[k] < dev->at[i] + N && dev->at[i] < dev->at[k] + N) return false;
-    }
-    return true;
-}
-
 template <typename real>
-static cudaError_t launch_init_as(dbm_t *h, const Fields5 &fields, int max_blocks, cudaStream_t s, int m0, int m1)
+static cudaError_t launch_init_as(dbm_t *h, const double *d_fields, cudaStream_t s, int m0, int m1)
 {
     double Fc[4][4];
     weight_coeffs(h->p.v, Fc);
     InitArgs<real> A;
     std::memset(&A, 0, sizeof(A));
-    for (int k = 0; k < 5; ++k) A.fields[k] = fields.at[k];
+    A.fields = d_fields;
     A.f = reinterpret_cast<real *>(h->buf + h->L.f[0]);
     A.lam = reinterpret_cast<real *>(h->buf + h->L.lam[0]);
     A.rowtab = reinterpret_cast<const real *>(h->buf + h->L.rowtab);
@@ -896,34 +844,34 @@ static cudaError_t launch_init_as(dbm_t *h, const Fields5 &fields, int max_block
         for (int c = 0; c < 4; ++c) A.Fc[k][c] = (real)Fc[k][c];
     }
     if constexpr (std::is_same<real, double>::value) static_cast<RingPowers<real> &>(A) = ring_powers(h->p.v);
-    return launch_init<real>(A, max_blocks, s);
+    return launch_init<real>(A, s);
 }
 
 extern "C" {
 
 // f = f^eq of the device fields into buffer 0 for theta rows [m0, m1); the
 // kernel checks every value and sets the handle's bad-input word.
-static int launch_init_rows(dbm_t *h, const Fields5 &fields, int max_blocks, cudaStream_t s, int m0, int m1)
+static int launch_init_rows(dbm_t *h, const double *d_fields, cudaStream_t s, int m0, int m1)
 {
-    const cudaError_t e = h->p.precision == DBM_FP64 ? launch_init_as<double>(h, fields, max_blocks, s, m0, m1)
-                                                     : launch_init_as<float>(h, fields, max_blocks, s, m0, m1);
+    const cudaError_t e = h->p.precision == DBM_FP64 ? launch_init_as<double>(h, d_fields, s, m0, m1)
+                                                     : launch_init_as<float>(h, d_fields, s, m0, m1);
     if (e != cudaSuccess) return cuda_fail(e, "init kernel launch");
     return DBM_OK;
 }
 
-static int launch_init_from(dbm_t *h, const Fields5 &fields, int max_blocks, cudaStream_t s)
+static int launch_init_from(dbm_t *h, const double *d_fields, cudaStream_t s)
 {
     CK(cudaMemsetAsync(bad_input_word(h), 0, sizeof(int), s));
-    const int rc = launch_init_rows(h, fields, max_blocks, s, 0, h->p.ntheta);
+    const int rc = launch_init_rows(h, d_fields, s, 0, h->p.ntheta);
     if (rc != DBM_OK) return rc;
     h->cur = 0;
     h->steps = 0;
     return DBM_OK;
 }
 
-// Theta-row chunks of the host-array calls on other memory: their copies
-// overlap the init or moments kernel of the neighbouring chunk, which runs on
-// the handle's second stream.  Small grids are one chunk.
+// Theta-row chunks of the host-array calls: their copies over the host link
+// (about 200 GB/s) overlap the init or moments kernel of the neighbouring
+// chunk, which runs on the handle's second stream.  Small grids are one chunk.
 static int host_chunks(const dbm_t *h)
 {
     const size_t bytes = (size_t)5 * h->p.nr * h->p.ntheta * sizeof(double);
@@ -937,24 +885,17 @@ int dbm_init_state(dbm_t *h, const double *rho, const double *ur, const double *
     const size_t N = (size_t)h->p.nr * h->p.ntheta;
     const int nr = h->p.nr, nth = h->p.ntheta;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    // Pinned fields are read by the init kernel where they are.  Others are
-    // staged in the second f buffer (free before the first step);
+    // Stage the fields in the second f buffer (free before the first step);
     // the init kernel validates them on the GPU, and one synchronisation at
     // the end covers the copies (the host arrays may be reused on return)
     // and the validation result.  Chunk c's copies go on `stream`, its init
     // kernel on the second stream once they have landed, while chunk c + 1
     // is copied.
     double *stage = reinterpret_cast<double *>(h->buf + h->L.f[1]);
-    const double *const src[5] = {rho, ur, uth, T, lam};
-    Fields5 pinned;
-    const bool direct = pinned_fields(src, N, &pinned);
-    if (direct) {
-        const int rc = launch_init_from(h, pinned, HOST_BLOCKS * h->nsm, s);
-        if (rc != DBM_OK) return rc;
-    }
-    const int C = direct ? 0 : host_chunks(h);
-    const int R = direct ? 0 : (nth + C - 1) / C;
-    if (!direct) CK(cudaMemsetAsync(bad_input_word(h), 0, sizeof(int), s));
+    const double *src[5] = {rho, ur, uth, T, lam};
+    const int C = host_chunks(h);
+    const int R = (nth + C - 1) / C;
+    CK(cudaMemsetAsync(bad_input_word(h), 0, sizeof(int), s));
     for (int c = 0; c < C; ++c) {
         const int m0 = c * R, m1 = std::min(nth, m0 + R);
         if (m0 >= m1) break;
@@ -967,7 +908,7 @@ int dbm_init_state(dbm_t *h, const double *rho, const double *ur, const double *
             CK(cudaStreamWaitEvent(h->aux, h->chunk_ev[c], 0));
             ks = h->aux;
         }
-        const int rc = launch_init_rows(h, planes(stage, N), INIT_BLOCKS, ks, m0, m1);
+        const int rc = launch_init_rows(h, stage, ks, m0, m1);
         if (rc != DBM_OK) return rc;
     }
     if (C > 1) {
@@ -987,7 +928,7 @@ int dbm_init_state_device(dbm_t *h, const double *d_fields, void *stream)
 {
     if (!h || !d_fields) return DBM_EINVAL;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const int rc = launch_init_from(h, planes(d_fields, (size_t)h->p.nr * h->p.ntheta), INIT_BLOCKS, s);
+    const int rc = launch_init_from(h, d_fields, s);
     if (rc == DBM_OK) note_work(h, s);
     return rc;
 }
@@ -1028,7 +969,7 @@ static cudaError_t launch_noneq_as(dbm_t *h, double *d_out, cudaStream_t s)
     MomArgs<real> A;
     std::memset(&A, 0, sizeof(A));
     A.f = reinterpret_cast<const real *>(h->buf + h->L.f[h->cur]);
-    A.out[0] = d_out;
+    A.out = d_out;
     A.plane = h->plane;
     A.nr = p.nr;
     A.ntheta = p.ntheta;
@@ -1047,7 +988,7 @@ static cudaError_t launch_noneq_as(dbm_t *h, double *d_out, cudaStream_t s)
 }
 
 template <typename real>
-static cudaError_t launch_moments_as(dbm_t *h, const Fields5 &out, double *partials, int grid, cudaStream_t s,
+static cudaError_t launch_moments_as(dbm_t *h, double *d_out, double *partials, int grid, cudaStream_t s,
                                      int m0, int m1)
 {
     const dbm_params &p = h->p;
@@ -1055,7 +996,7 @@ static cudaError_t launch_moments_as(dbm_t *h, const Fields5 &out, double *parti
     std::memset(&A, 0, sizeof(A));
     A.f = reinterpret_cast<const real *>(h->buf + h->L.f[h->cur]);
     A.lam = reinterpret_cast<const real *>(h->buf + h->L.lam[h->cur]);
-    for (int k = 0; k < 5; ++k) A.out[k] = out.at[k];
+    A.out = d_out;
     A.partials = partials;
     A.status = reinterpret_cast<int *>(h->buf + h->L.status);
     A.rowtab = reinterpret_cast<const real *>(h->buf + h->L.rowtab);
@@ -1077,16 +1018,16 @@ static cudaError_t launch_moments_as(dbm_t *h, const Fields5 &out, double *parti
 
 extern "C" {
 
-// Moments of theta rows [m0, m1) into `out`, their per-block partial sums at
+// Moments of theta rows [m0, m1) into d_out, their per-block partial sums at
 // partial slot *slot0 onwards (advanced past them), at most max_blocks blocks.
-static int launch_moments_rows(dbm_t *h, const Fields5 &out, cudaStream_t s, int m0, int m1, int max_blocks,
+static int launch_moments_rows(dbm_t *h, double *d_out, cudaStream_t s, int m0, int m1, int max_blocks,
                                int *slot0)
 {
     const long long n = (long long)h->p.nr * (m1 - m0);
     const int grid = (int)std::max<long long>(1, std::min<long long>((n + 255) / 256, max_blocks));
     double *partials = reinterpret_cast<double *>(h->buf + h->L.partials) + (size_t)*slot0 * 4;
-    const cudaError_t e = h->p.precision == DBM_FP64 ? launch_moments_as<double>(h, out, partials, grid, s, m0, m1)
-                                                     : launch_moments_as<float>(h, out, partials, grid, s, m0, m1);
+    const cudaError_t e = h->p.precision == DBM_FP64 ? launch_moments_as<double>(h, d_out, partials, grid, s, m0, m1)
+                                                     : launch_moments_as<float>(h, d_out, partials, grid, s, m0, m1);
     if (e != cudaSuccess) return cuda_fail(e, "moments kernel launch");
     *slot0 += grid;
     return DBM_OK;
@@ -1103,8 +1044,7 @@ static int launch_totals_of(dbm_t *h, int nblocks, cudaStream_t s)
 static int launch_moments_into(dbm_t *h, double *d_out, cudaStream_t s)
 {
     int nblocks = 0;
-    int rc = launch_moments_rows(h, planes(d_out, (size_t)h->p.nr * h->p.ntheta), s, 0, h->p.ntheta,
-                                 std::min(MOMENT_BLOCKS, 4 * h->nsm), &nblocks);
+    int rc = launch_moments_rows(h, d_out, s, 0, h->p.ntheta, std::min(MOMENT_BLOCKS, 4 * h->nsm), &nblocks);
     if (rc != DBM_OK) return rc;
     return launch_totals_of(h, nblocks, s);
 }
@@ -1158,21 +1098,15 @@ int dbm_moments(dbm_t *h, double *rho, double *ur, double *uth, double *T, doubl
     const int nr = h->p.nr, nth = h->p.ntheta;
     double *stage = reinterpret_cast<double *>(h->buf + h->L.f[1 - h->cur]);
     double *dst[5] = {rho, ur, uth, T, lam};
-    int nblocks = 0, rc = DBM_OK;
-    Fields5 pinned;
-    const bool direct = pinned_fields({rho, ur, uth, T, lam}, N, &pinned);
-    if (direct) {  // the moments kernel writes them where they are
-        rc = launch_moments_rows(h, pinned, s, 0, nth, std::min(MOMENT_BLOCKS, HOST_BLOCKS * h->nsm), &nblocks);
-        if (rc != DBM_OK) return rc;
-    }
     // Chunk c's moments kernel on `stream`; its copies to the host arrays on
     // the second stream once it is done, while chunk c + 1 is computed.
-    const int C = direct ? 0 : host_chunks(h);
-    const int R = direct ? 0 : (nth + C - 1) / C;
+    const int C = host_chunks(h);
+    const int R = (nth + C - 1) / C;
+    int nblocks = 0;
     for (int c = 0; c < C; ++c) {
         const int m0 = c * R, m1 = std::min(nth, m0 + R);
         if (m0 >= m1) break;
-        rc = launch_moments_rows(h, planes(stage, N), s, m0, m1, MOMENT_BLOCKS / C, &nblocks);
+        int rc = launch_moments_rows(h, stage, s, m0, m1, MOMENT_BLOCKS / C, &nblocks);
         if (rc != DBM_OK) return rc;
         cudaStream_t cs = s;
         if (C > 1) {
@@ -1185,7 +1119,7 @@ int dbm_moments(dbm_t *h, double *rho, double *ur, double *uth, double *T, doubl
             if (dst[f])
                 CK(cudaMemcpyAsync(dst[f] + off, stage + f * N + off, cnt * sizeof(double), cudaMemcpyDeviceToHost, cs));
     }
-    rc = launch_totals_of(h, nblocks, s);
+    int rc = launch_totals_of(h, nblocks, s);
     if (rc != DBM_OK) return rc;
     if (totals)
         CK(cudaMemcpyAsync(totals, h->buf + h->L.totals, 4 * sizeof(double), cudaMemcpyDeviceToHost, s));

@@ -1299,7 +1299,7 @@ static __global__ void rcp_selftest_kernel(const float *x, float *approx, float 
 // ---------------------------------------------------------------------------
 template <typename real>
 struct InitArgs : RingPowers<real> {
-    const double *fields[5];  // rho, ur, uth, T, lambda; device memory or pinned host memory
+    const double *fields;
     real *f;
     real *lam;
     const real *rowtab;  // [ntheta][16]: cos, sin of (i pi/4 - theta_m)
@@ -1317,12 +1317,13 @@ __global__ void __launch_bounds__(256) init_kernel(const InitArgs<real> A)
     using O = Op<real>;
     const real H = real(0.70710678118654752440);
     const real one = real(1), half = real(0.5);
+    const long long N = (long long)A.nr * A.ntheta;
     bool bad = false;
     for (long long s = (long long)A.m0 * A.nr + blockIdx.x * (long long)blockDim.x + threadIdx.x;
          s < (long long)A.m1 * A.nr; s += (long long)gridDim.x * blockDim.x) {
         const int m = (int)(s / A.nr), j = (int)(s - (long long)m * A.nr);
-        const double rho_d = A.fields[0][s], ur_d = A.fields[1][s], uth_d = A.fields[2][s];
-        const double T_d = A.fields[3][s], lam_d = A.fields[4][s];
+        const double rho_d = A.fields[s], ur_d = A.fields[N + s], uth_d = A.fields[2 * N + s];
+        const double T_d = A.fields[3 * N + s], lam_d = A.fields[4 * N + s];
         if (!(rho_d > 0.0) || !(T_d > 0.0) || !isfinite(rho_d) || !isfinite(T_d) || !isfinite(ur_d) ||
             !isfinite(uth_d) || !isfinite(lam_d)) {
             bad = true;
@@ -1444,8 +1445,7 @@ template <typename real>
 struct MomArgs {
     const real *f;
     const real *lam;
-    double *out[5];      // rho, ur, uth, T, lambda (any may be null; device memory or pinned host
-                         // memory); the non-equilibrium moments' 12 planes
+    double *out;
     double *partials;
     int *status;
     const real *rowtab;  // [ntheta][16] (moments)
@@ -1478,6 +1478,7 @@ __device__ __forceinline__ double warp_sum4(const double (&v)[4], int lane)
 template <typename real>
 __global__ void __launch_bounds__(MOMENT_THREADS) moments_kernel(const MomArgs<real> A)
 {
+    const long long N = (long long)A.nr * A.ntheta;
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
     bool bad = false;
     if constexpr (sizeof(real) == 4) {
@@ -1501,11 +1502,13 @@ __global__ void __launch_bounds__(MOMENT_THREADS) moments_kernel(const MomArgs<r
             // conversions by integer shifts: each would cost an FP64 instruction, and
             // those, 16 per site with them and 7 without, would take the time
             const float y = A.lam[(long long)m * A.ld + j];
-            if (A.out[0]) A.out[0][s] = widen(rho);
-            if (A.out[1]) A.out[1][s] = widen(ur);
-            if (A.out[2]) A.out[2][s] = widen(uth);
-            if (A.out[3]) A.out[3][s] = widen(T);
-            if (A.out[4]) A.out[4][s] = LamStore<float>::to_lambda(widen(y));
+            if (A.out) {
+                A.out[s] = widen(rho);
+                A.out[N + s] = widen(ur);
+                A.out[2 * N + s] = widen(uth);
+                A.out[3 * N + s] = widen(T);
+                A.out[4 * N + s] = LamStore<float>::to_lambda(widen(y));
+            }
             bad |= !isfinite(rho) || !isfinite(ur) || !isfinite(uth) || !isfinite(T) || !isfinite(y);
             // weight r dr dtheta: dr dtheta applied per block; j + 1/2 from the bits of 2^52 + j
             const double r = fma(__hiloint2double(0x43300000, j) - 4503599627370495.5, A.dr, A.r_in);
@@ -1536,11 +1539,13 @@ __global__ void __launch_bounds__(MOMENT_THREADS) moments_kernel(const MomArgs<r
             const double cth = A.rowtab[(long long)m * 16], sth = -A.rowtab[(long long)m * 16 + 8];
             const double ur = fma(ux, cth, uy * sth), uth = fma(uy, cth, -(ux * sth));
             const double lam = LamStore<real>::to_lambda((double)A.lam[(long long)m * A.ld + j]);
-            if (A.out[0]) A.out[0][s] = rho;
-            if (A.out[1]) A.out[1][s] = ur;
-            if (A.out[2]) A.out[2][s] = uth;
-            if (A.out[3]) A.out[3][s] = T;
-            if (A.out[4]) A.out[4][s] = lam;
+            if (A.out) {
+                A.out[s] = rho;
+                A.out[N + s] = ur;
+                A.out[2 * N + s] = uth;
+                A.out[3 * N + s] = T;
+                A.out[4 * N + s] = lam;
+            }
             bad |= !isfinite(rho) || !isfinite(ur) || !isfinite(uth) || !isfinite(T) || !isfinite(lam);
             const double r = A.r_in + (j + 0.5) * A.dr;  // weight r dr dtheta: dr dtheta applied per block
             acc[0] = fma(rho, r, acc[0]);
@@ -1657,7 +1662,7 @@ __global__ void __launch_bounds__(256) noneq_kernel(const MomArgs<real> A)
             const double f_rt = fma(-UV, z, 0.5 * Y4) - fma(V, h_r, U * h_t) - 2.0 * fma(U, rrt, V * rtt) - u2 * rt;
             // less the Maxwellian's: rho T = half the trace, 2 rho T^2
             const double rT = 0.5 * tr, rTT2 = 2.0 * rT * (rT * inv_rho);
-            double *out = A.out[0] + s;
+            double *out = A.out + s;
             out[0] = rr - rT;
             out[N] = rt;
             out[2 * N] = tt - rT;

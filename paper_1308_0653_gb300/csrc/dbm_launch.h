@@ -49,7 +49,7 @@ cudaError_t launch_batch_advance(long long *T, int k, cudaStream_t s);
 template <typename real> int batch_const_capacity();
 template <typename real>
 cudaError_t upload_batch_consts(int first, const StepConsts<real> *src, int n, cudaStream_t s);
-template <typename real> cudaError_t launch_init(const InitArgs<real> &A, int max_blocks, cudaStream_t s);
+template <typename real> cudaError_t launch_init(const InitArgs<real> &A, cudaStream_t s);
 template <typename real> cudaError_t launch_moments(const MomArgs<real> &A, int grid, cudaStream_t s);
 template <typename real> cudaError_t launch_noneq(const MomArgs<real> &A, int grid, cudaStream_t s);
 cudaError_t launch_totals(const double *partials, int nblocks, double *totals, cudaStream_t s);
