@@ -172,8 +172,7 @@ int dbm_destroy(dbm_t *h);
  * (Eq. feq, Sec. II.B) of the fields at every site, lambda copied (reading:
  * the paper gives macroscopic initial data only).  f^eq is evaluated in the
  * state's precision with the arithmetic of the step's own equilibrium.  The
- * fields are read by the init kernel, pinned ones where they are, others
- * after a copy to the device, and checked there;
+ * fields are copied to the device and checked there by the init kernel;
  * the call synchronises `stream` once at the end, so the host arrays may be
  * reused on return.  Resets the step counter.
  * Errors: DBM_EINVAL (NULL array, or some rho <= 0, T <= 0 or non-finite
@@ -193,8 +192,8 @@ int dbm_init_state_device(dbm_t *h, const double *d_fields, void *stream);
  * step kernel for long runs.  Errors: DBM_EINVAL (nsteps < 0), DBM_ECUDA. */
 int dbm_step(dbm_t *h, int64_t nsteps, void *stream);
 
-/* Macroscopic fields of the current state, written to host arrays (any may be
- * NULL; pinned ones by the moments kernel itself, others copied): rho = sum f, u = sum f v / rho in polar components, T = sum f
+/* Macroscopic fields of the current state, copied to host arrays (any may be
+ * NULL): rho = sum f, u = sum f v / rho in polar components, T = sum f
  * (v - u)^2 / (2 rho) (Sec. II.B), lambda.  Each site's moments are
  * evaluated in the state's precision: FP64 states in FP64; FP32 states in
  * FP32 ring by ring, the very values the step computes, widened to double.
