@@ -284,6 +284,13 @@ int dbm_selftest_rcp(const float *d_x, float *d_approx, float *d_ieee, int n, vo
  * Errors: DBM_EINVAL, DBM_ECUDA. */
 int dbm_selftest_wait(int *d_status, int arrive, int64_t limit_cycles, void *stream);
 
+/* Checked builds only (DBM_EINVAL otherwise): the row ring of this handle, alone
+ * or attached to a batch after this call, loads at most `rows` rows per CTA and
+ * step (0: all), so that the waits for the others run out (after about a second)
+ * and the step ends through its abort path: dbm_status then is DBM_ETIMEOUT and
+ * the state undefined. */
+int dbm_selftest_stop_loads(dbm_t *h, int rows);
+
 /* Number of step-kernel variants for a precision (0 if invalid).  Variants
  * differ only in how the work is staged (pipeline, ring depth, registers);
  * every variant computes the same update bit for bit. */

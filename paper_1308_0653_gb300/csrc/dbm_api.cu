@@ -196,6 +196,7 @@ struct dbm_s {
     int device;
     bool tmap_ok;             // tensor maps encoded (tensor-TMA variants usable)
     cudaEvent_t done;         // recorded after the last work that touches the buffers
+    int stop_loads;           // checked builds: see dbm_selftest_stop_loads
     int host_word[2];         // host side of small device-to-host status copies
     cudaStream_t aux;         // second stream of the chunked host-array calls
     cudaEvent_t chunk_ev[4], join_ev;
@@ -304,6 +305,9 @@ void fill_step_args(dbm_t *h, StepArgs<real> (&a)[2])
         A.rows_per_item = h->rows_per_item;
         A.segs = (p.ntheta + h->rows_per_item - 1) / h->rows_per_item;
         A.items = A.strips * A.segs;
+#ifdef DBM_DEBUG
+        A.stop_loads = h->stop_loads;
+#endif
         A.c.reaction_energy = p.reaction_energy;
         A.c.general_pow = (p.m == 1.0 && p.n == 1.0) ? 0 : 1;
         A.c.sector = p.sector;
@@ -1223,6 +1227,17 @@ int dbm_selftest_wait(int *d_status, int arrive, int64_t limit_cycles, void *str
                                          static_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) return cuda_fail(e, "wait self-test launch");
     return DBM_OK;
+}
+
+int dbm_selftest_stop_loads(dbm_t *h, int rows)
+{
+    if (!h || rows < 0) return DBM_EINVAL;
+#ifdef DBM_DEBUG
+    h->stop_loads = rows;
+    return configure_launch(h, h->variant);
+#else
+    return DBM_EINVAL;
+#endif
 }
 
 int dbm_num_variants(int precision)

@@ -41,16 +41,27 @@ constexpr int ST_BOUNDS = 8;         // DBM_DEBUG builds: a copy or store failed
 // the row and 16-byte aligned) and every global store of the update, and skip
 // a failing one with ST_BOUNDS set; a skipped copy ends the step through the
 // abort path, like an expired wait.  Release builds compile the checks out.
+// Code whose warps vote or shuffle further on asks by whole warps (_WARP): a
+// lane that left alone would be waited for.
 #ifdef DBM_DEBUG
 #define DBM_DEBUG_CHECK(cond, status_ptr) (dbm::debug_check((cond), (status_ptr)))
+#define DBM_DEBUG_CHECK_WARP(cond, status_ptr) (!dbm::warp_any(!dbm::debug_check((cond), (status_ptr))))
 #else
 #define DBM_DEBUG_CHECK(cond, status_ptr) (true)
+#define DBM_DEBUG_CHECK_WARP(cond, status_ptr) (true)
 #endif
 __device__ __forceinline__ bool debug_check(bool ok, int *status)
 {
     if (!ok) atomicOr(status, ST_BOUNDS);
     return ok;
 }
+
+// Whether x holds in any lane, asked by all 32: the same answer in each.  What
+// ends a step early (an expired wait, the abort flag that another warp may be
+// setting) is decided by it, or by the whole block: lanes that each made up
+// their own mind could part, and those that went on would wait for the others
+// in the next vote, shuffle or warp barrier without end.
+__device__ __forceinline__ bool warp_any(bool x) { return __any_sync(0xffffffffu, x); }
 
 template <typename real> struct Halo;
 template <> struct Halo<float> { static constexpr int value = 4; };   // 16 bytes
@@ -105,6 +116,9 @@ struct StepArgs {
     int rows_per_item;    // theta rows per work item
     int segs;             // ceil(ntheta / rows_per_item)
     int items;            // strips * segs
+#ifdef DBM_DEBUG
+    int stop_loads;       // > 0: a CTA's producer stops after that many rows (dbm_selftest_stop_loads)
+#endif
     StepConsts<real> c;
 };
 
@@ -557,14 +571,17 @@ __device__ __forceinline__ bool upwind_below(const float (&c)[4], int i)
 // col is the site's column.  A row's directions share their signs and a site
 // its two radial neighbours, so a neighbour is one select; only a sector's disc
 // centre and first and last row turn the velocity set.
-template <int WP, int LAMOFF, typename Put>
-__device__ __forceinline__ void ring_site_update(const StepArgs<float> &A, const StepConsts<float> &C,
+// WHOLE: called by whole warps that vote in `put`; false where a check failed
+// and nothing was put.
+template <int WP, int LAMOFF, bool WHOLE, typename Put>
+__device__ __forceinline__ bool ring_site_update(const StepArgs<float> &A, const StepConsts<float> &C,
                                                  const float *__restrict__ sp, const float *__restrict__ sc,
                                                  const float *__restrict__ sn, int col, int j, int m, float inv_r,
                                                  const float (&cs)[4], const float (&sn4)[4], bool active, Put put)
 {
     // the site's stores stay inside its instance's planes
-    if (!DBM_DEBUG_CHECK(j >= 0 && (j < A.nr || !active) && A.nr <= A.ld && m >= 0 && m < A.ntheta, A.status)) return;
+    bool ok = DBM_DEBUG_CHECK(j >= 0 && (j < A.nr || !active) && A.nr <= A.ld && m >= 0 && m < A.ntheta, A.status);
+    if (!(WHOLE ? DBM_DEBUG_CHECK_WARP(ok, A.status) : ok)) return false;
     float f[NV];
 #pragma unroll
     for (int q = 0; q < NV; ++q) f[q] = sc[q * WP + col];
@@ -592,16 +609,17 @@ __device__ __forceinline__ void ring_site_update(const StepArgs<float> &A, const
         // velocity planes q = 1 + i .. 25 + i of direction i: neighbour reads
         // stay inside the 33 planes of their row buffer
         const int r = (int)(rn[i] - sc), t = (int)(tn[i] - (upwind_below(sn4, i) ? sp : sn));
-        const bool ok = (1 + i) * WP + r >= 0 && (25 + i) * WP + r < NV * WP && (1 + i) * WP + t >= 0 &&
-                        (25 + i) * WP + t < NV * WP;
-        if (!DBM_DEBUG_CHECK(ok, A.status)) return;
+        ok = ok && (1 + i) * WP + r >= 0 && (25 + i) * WP + r < NV * WP && (1 + i) * WP + t >= 0 &&
+             (25 + i) * WP + t < NV * WP;
     }
+    if (!(WHOLE ? DBM_DEBUG_CHECK_WARP(ok, A.status) : DBM_DEBUG_CHECK(ok, A.status))) return false;
 #endif
     const float ln = site_update(
         C, f, sc[LAMOFF + col], A.ld, j, m, inv_r, cs, sn4, [&](int q, int i) { return rn[i][q * WP]; },
         [&](int q, int i) { return tn[i][q * WP]; }, put, [&](bool inner) { return (inner ? left : right)[LAMOFF]; },
         [&](bool below) { return (below ? prev : next)[LAMOFF]; });
     if (active) A.lam_out[(long long)m * A.ld + j] = ln;
+    return true;
 }
 
 }  // namespace dbm
@@ -785,7 +803,11 @@ __device__ __forceinline__ void march(const Work &work, unsigned char *smem_raw,
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
         const StepArgs<real> *a;
         int j0, mb, me, cidx;
-        if (work.item(it, a, j0, mb, me, cidx)) total_loads += (me - mb) + 2;
+        if (!work.item(it, a, j0, mb, me, cidx)) continue;
+        total_loads += (me - mb) + 2;
+#ifdef DBM_DEBUG
+        if (a->stop_loads > 0) total_loads = min(total_loads, (long long)a->stop_loads);
+#endif
     }
 
     // Producer cursor (replicated in the lanes of warp 0).
@@ -852,17 +874,19 @@ __device__ __forceinline__ void march(const Work &work, unsigned char *smem_raw,
         for (int c = 1; c <= L; ++c) {
             const long long P = base + c;
             // wait for rows at positions P-1, P, P+1
+            bool late = false;
 #pragma unroll
             for (int d = -1; d <= 1; ++d) {
                 const long long Q = P + d;
-                if (!mbar_wait_bounded(&bars[Q % NSTAGE], (uint32_t)((Q / NSTAGE) & 1))) {
-                    atomicOr(A.status, ST_WAIT_TIMEOUT);
-                    abort_flag = 1;
-                }
+                late = late || !mbar_wait_bounded(&bars[Q % NSTAGE], (uint32_t)((Q / NSTAGE) & 1));
+            }
+            if (late) {
+                atomicOr(A.status, ST_WAIT_TIMEOUT);
+                abort_flag = 1;
             }
             const int m = mb + c - 1;
             if constexpr (sizeof(real) == 8) {  // every lane takes part (idle ones store nothing)
-                if (!abort_flag) {
+                if (!warp_any(late)) {
                     const bool ghost = C.centre == 2 && j == 0;
                     if (ghost) fill_centre_ghost<real, WP, NV * WP, HALO>(A, sm + (P % NSTAGE) * SLOT, m);
                     __syncwarp();
@@ -871,7 +895,7 @@ __device__ __forceinline__ void march(const Work &work, unsigned char *smem_raw,
                                                           j0, tx, m, A.rowtab + (long long)m * 16);
                     if (ghost) fence_proxy_async_smem();
                 }
-            } else if (active && !abort_flag) {
+            } else if (active && !late) {
                 real cs[4], sn4[4];
                 const real *rt = A.rowtab + (long long)m * 16;
 #pragma unroll
@@ -882,13 +906,12 @@ __device__ __forceinline__ void march(const Work &work, unsigned char *smem_raw,
                 const bool ghost = C.centre == 2 && j == 0;
                 if (ghost) fill_centre_ghost<real, WP, NV * WP, HALO>(A, sm + (P % NSTAGE) * SLOT, m);
                 real *out = A.f_out + (long long)m * A.ld + j;
-                ring_site_update<WP, NV * WP>(A, C, sm + ((P - 1) % NSTAGE) * SLOT, sm + (P % NSTAGE) * SLOT,
+                ring_site_update<WP, NV * WP, false>(A, C, sm + ((P - 1) % NSTAGE) * SLOT, sm + (P % NSTAGE) * SLOT,
                                          sm + ((P + 1) % NSTAGE) * SLOT, HALO + tx, j, m, inv_r, cs, sn4, true,
                                          [&](int q, float v) { out[(long long)q * A.plane] = v; });
                 if (ghost) fence_proxy_async_smem();
             }
-            __syncthreads();
-            if (abort_flag) {
+            if (__syncthreads_or(*(volatile int *)&abort_flag)) {  // the block's answer
                 ok = false;
                 break;
             }
@@ -1012,7 +1035,11 @@ __device__ __forceinline__ void march2(const Work &work, unsigned char *smem_raw
         for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
             const StepArgs<real> *a;
             int j0, mb, me, cidx;
-            if (work.item(it, a, j0, mb, me, cidx)) total_loads += (me - mb) + 2;
+            if (!work.item(it, a, j0, mb, me, cidx)) continue;
+            total_loads += (me - mb) + 2;
+#ifdef DBM_DEBUG
+            if (a->stop_loads > 0) total_loads = min(total_loads, a->stop_loads);
+#endif
         }
         int issued = 0;
         int p_item = blockIdx.x, p_row = 0;
@@ -1028,12 +1055,11 @@ __device__ __forceinline__ void march2(const Work &work, unsigned char *smem_raw
             if (issued >= NSTAGE) {
                 const uint32_t par = (uint32_t)((issued / NSTAGE - 1) & 1);
                 if (!mbar_wait_bounded(&empty[slot], par)) {
-                    if (lane == 0) atomicOr(pa->status, ST_WAIT_TIMEOUT);
+                    atomicOr(pa->status, ST_WAIT_TIMEOUT);
                     abort_flag = 1;
                 }
             }
-            __syncwarp();
-            if (*(volatile int *)&abort_flag) break;
+            if (warp_any(*(volatile int *)&abort_flag)) break;
             int m = pmb - 1 + p_row;
             const int nth = pa->ntheta;
             m = m < 0 ? m + nth : (m >= nth ? m - nth : m);
@@ -1103,18 +1129,19 @@ __device__ __forceinline__ void march2(const Work &work, unsigned char *smem_raw
         real *stage = sm + NSTAGE * SLOT + warp * (NV * 32);  // STAGE: this warp's outgoing row
         // Ring position taken next: slot and phase parity.  A wait, even for a row
         // that has landed, takes some 150 cycles, so each row asks for the next
-        // one's barrier in the middle of its own arithmetic (`landed`).
+        // one's barrier in the middle of its own arithmetic (`landed`, this lane's
+        // answer; the warp's is voted when the position is taken).
         int slot = 0;
         uint32_t phase = 0;
         bool landed = false;
         auto ask = [&]() { landed = mbar_test_wait(&full[slot], phase); };
         auto take = [&](const StepArgs<real> &A) -> int {
-            if (!landed) {
+            if (warp_any(!landed)) {
                 if (!mbar_wait_bounded(&full[slot], phase)) {
-                    if (lane == 0) atomicOr(A.status, ST_WAIT_TIMEOUT);
+                    atomicOr(A.status, ST_WAIT_TIMEOUT);
                     abort_flag = 1;
                 }
-                if (*(volatile int *)&abort_flag) ok = false;
+                if (warp_any(*(volatile int *)&abort_flag)) ok = false;
             }
             landed = false;
             const int taken = slot;
@@ -1156,26 +1183,26 @@ __device__ __forceinline__ void march2(const Work &work, unsigned char *smem_raw
                     }
                     if (ghost) fill_centre_ghost<real, WP, LAMOFF, HALO>(A, sc, m);
                     if constexpr (STAGE) {
-                        ring_site_update<WP, LAMOFF>(A, C, sp, sc, sn, HALO + tx, j, m, inv_r, cs, sn4, active,
-                                                     [&](int q, float v) {
-                                                         if (q == 0) {
-                                                             ask();
-                                                             // the store before has read the staging row
-                                                             if (lane == 0) bulk_wait_read();
-                                                             __syncwarp();
-                                                         }
-                                                         stage[q * 32 + lane] = v;
-                                                     });
+                        const bool put = ring_site_update<WP, LAMOFF, true>(
+                            A, C, sp, sc, sn, HALO + tx, j, m, inv_r, cs, sn4, active, [&](int q, float v) {
+                                if (q == 0) {
+                                    ask();
+                                    // the store before has read the staging row
+                                    if (lane == 0) bulk_wait_read();
+                                    __syncwarp();
+                                }
+                                stage[q * 32 + lane] = v;
+                            });
                         fence_proxy_async_smem();
                         __syncwarp();
-                        if (lane == 0 && (Work::kCopyArgs || j < A.nr)) {
+                        if (put && lane == 0 && (Work::kCopyArgs || j < A.nr)) {
                             tma_store_3d(out_map, stage, j, m, 0);
                             bulk_commit();
                         }
                     } else {
                         real *out = A.f_out + (long long)m * A.ld + j;
-                        ring_site_update<WP, LAMOFF>(A, C, sp, sc, sn, HALO + tx, j, m, inv_r, cs, sn4, true,
-                                                     [&](int q, float v) { out[(long long)q * A.plane] = v; });
+                        ring_site_update<WP, LAMOFF, false>(A, C, sp, sc, sn, HALO + tx, j, m, inv_r, cs, sn4, true,
+                                                            [&](int q, float v) { out[(long long)q * A.plane] = v; });
                         if (ghost) fence_proxy_async_smem();
                     }
                 }
@@ -1191,7 +1218,10 @@ __device__ __forceinline__ void march2(const Work &work, unsigned char *smem_raw
                 s_cur = s_next;
             }
         };
-        for (int it = blockIdx.x; it < nitems && ok; it += gridDim.x) {
+        // After an expired wait a batch's warps still go through the items: the
+        // barrier of each counts all of them, and one may be an item ahead of the
+        // one that gave up.
+        for (int it = blockIdx.x; it < nitems && (ok || Work::kCopyArgs); it += gridDim.x) {
             const StepArgs<real> *ga;
             int j0, mb, me, cidx;
             if (!work.item(it, ga, j0, mb, me, cidx)) continue;
@@ -1205,6 +1235,7 @@ __device__ __forceinline__ void march2(const Work &work, unsigned char *smem_raw
                     reinterpret_cast<int *>(dst)[q] = reinterpret_cast<const int *>(ga)[q];
                 named_bar_sync(1, W);
                 parity ^= 1;
+                if (!ok) continue;
                 if (STAGE && lane == 0) fence_tensormap_acquire(&ga->tm_out);
                 // The item's pointers and sizes from there into registers for
                 // the item (a single instance reads its constants from the

@@ -33,7 +33,7 @@ template <int G, bool AHEAD, typename Args>
 __device__ __forceinline__ void direct64_task(const Args &A, const StepConsts<double> &C, int row, int j_raw)
 {
     const int j = min(j_raw, A.nr - 1), m = row;
-    if (!DBM_DEBUG_CHECK(j >= 0 && m >= 0 && m < A.ntheta && A.nr <= A.ld, A.status)) return;
+    if (!DBM_DEBUG_CHECK_WARP(j >= 0 && m >= 0 && m < A.ntheta && A.nr <= A.ld, A.status)) return;
     const int mp = m == 0 ? A.ntheta - 1 : m - 1, mn = m == A.ntheta - 1 ? 0 : m + 1;
     const long long at = (long long)m * A.ld + j, dp = (long long)(mp - m) * A.ld, dn = (long long)(mn - m) * A.ld;
     long long dl = j > 0 ? -1 : 0;

@@ -287,7 +287,7 @@ __device__ __forceinline__ void site_update64_ring(const StepArgs<double> &A, co
                                                    int tx, int m, const double *rt)
 {
     const int j = min(j0 + tx, A.nr - 1), col = HALO + j - j0;
-    if (!DBM_DEBUG_CHECK(j >= 0 && A.nr <= A.ld && m >= 0 && m < A.ntheta && col >= 1 && col + 1 < WP, A.status))
+    if (!DBM_DEBUG_CHECK_WARP(j >= 0 && A.nr <= A.ld && m >= 0 && m < A.ntheta && col >= 1 && col + 1 < WP, A.status))
         return;
     const int left = col - (j > 0 || C.centre == 2 ? 1 : 0), right = col + (j < A.nr - 1 ? 1 : 0);
     const Places64 p{sc + col,          sc + left,          sc + right,          sp + col,          sn + col,
