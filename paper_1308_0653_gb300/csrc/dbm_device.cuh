@@ -1469,7 +1469,12 @@ __device__ __forceinline__ RingHarmonics ring_harmonics(const double (&g)[8])
 // carries ~6e-8 relative rounding per value, so FP64 per-site arithmetic would
 // add no accuracy).  The FP64 kernel is bound by its FP64 instructions: about
 // 110 per site this way, 369 with per-velocity sums, a second pass for T and
-// the row's angle evaluated at every site.
+// the row's angle evaluated at every site.  FP64's T = (sum f v^2 / rho - u^2) / 2
+// loses digits to the subtraction as u grows; from about u^2 = 1.5 T on a second pass
+// is the more exact (rms error, states within 5 % of f^eq at T = 1: 1.5e-16
+// against 2.6e-16 at u = 0.5, 2.6 against 2.7 at 1.25, 7.2 against 4.3 at 2; a
+// second pass velocity by velocity 3.4, 3.5 and 4.7), so those sites take it
+// (2048^2: 0.84 ms without, 1.64 with every site in it).
 // out: [5][ntheta][nr] doubles; partials: [gridDim.x][4] (scratch).
 // ---------------------------------------------------------------------------
 template <typename real>
@@ -1504,6 +1509,26 @@ __device__ __forceinline__ double warp_sum4(const double (&v)[4], int lane)
     double k = (odd ? k1 : k0) + __shfl_xor_sync(ALL, odd ? k0 : k1, 8);
     for (int o = 4; o > 0; o >>= 1) k += __shfl_xor_sync(ALL, k, o);
     return k;
+}
+
+// T = sum f |v - u|^2 / (2 rho) of an FP64 site in which the flow is fast, from
+// its f once more: with w_i = e_i . u, |v_k e_i - u|^2 = (v_k - w_i)^2 + w_{i+2}^2.
+__device__ __forceinline__ double peculiar_T(const double *fp, long long plane, const double (&v)[4], double ux,
+                                             double uy, double inv_rho)
+{
+    const double H = 0.70710678118654752440;
+    const double w[4] = {ux, H * (ux + uy), uy, H * (uy - ux)};
+    double e = fp[0] * fma(ux, ux, uy * uy);
+#pragma unroll 1
+    for (int k = 0; k < 4; ++k) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const double w2 = w[(i + 2) & 3] * w[(i + 2) & 3], a = v[k] - w[i], b = v[k] + w[i];
+            e = fma(fp[(1 + 8 * k + i) * plane], fma(a, a, w2), e);
+            e = fma(fp[(5 + 8 * k + i) * plane], fma(b, b, w2), e);
+        }
+    }
+    return 0.5 * (e * inv_rho);
 }
 
 template <typename real>
@@ -1566,7 +1591,10 @@ __global__ void __launch_bounds__(MOMENT_THREADS) moments_kernel(const MomArgs<r
             ring_moments<real>(fv, A.vr, A.v2r, rho, jx, jy, e2);
             const double inv_rho = 1.0 / rho;
             const double ux = jx * inv_rho, uy = jy * inv_rho;
-            const double T = 0.5 * fma(e2, inv_rho, -fma(ux, ux, uy * uy));
+            const double u2 = fma(ux, ux, uy * uy);
+            double T = 0.5 * fma(e2, inv_rho, -u2);
+            // by the upper words, FP64 instructions being what this kernel costs: u^2 > 1.25 to 1.5 T
+            if (__double2hiint(u2) > __double2hiint(T) + 0x80000) T = peculiar_T(fp, A.plane, A.vr, ux, uy, inv_rho);
             const double cth = A.rowtab[(long long)m * 16], sth = -A.rowtab[(long long)m * 16 + 8];
             const double ur = fma(ux, cth, uy * sth), uth = fma(uy, cth, -(ux * sth));
             const double lam = LamStore<real>::to_lambda((double)A.lam[(long long)m * A.ld + j]);
