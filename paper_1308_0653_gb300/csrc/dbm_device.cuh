@@ -1642,6 +1642,60 @@ __global__ void __launch_bounds__(MOMENT_THREADS) moments_kernel(const MomArgs<r
 // then made central with u.  About 240 FP64 instructions per site where the
 // 33 x 12 direct sums took 1180.  The row's angles are evaluated once per
 // block and row.
+//
+// What u contributes to raw moments is taken off again with its rounding: that
+// of Delta*_2's r-theta part, the smallest, passes that of sums over v - u first,
+// by 1.3 at u^2 = T / 4 (all others at 0.5 to 1 times theirs) and all of them by
+// 2 to 3 at u = 2, T = 1.6.  FP64 sites beyond u^2 = T / 4 take those sums
+// (2048^2: 1.90 ms without, 6.0 where every site does; 9.2 with the 33 x 12 sums).
+// FP32 states carry 1e9 times that rounding in f and don't.
+
+// Delta* by sums over v - u of an FP64 site's f (about 630 FP64 instructions).
+// t: cos, sin of theta; U, V: u in the polar frame.
+template <typename real>
+__device__ __forceinline__ void central_sums(const real *fp, long long plane, const double (&v)[4], double U,
+                                             double V, const double *t, double inv_rho, double *out, long long N)
+{
+    const double H = 0.70710678118654752440, c = t[0], s = t[1];
+    const double ex[4] = {c, H * (c + s), s, H * (s - c)}, ey[4] = {-s, H * (c - s), c, H * (c + s)};
+    double rr = 0.0, rt = 0.0, tt = 0.0, rrr = 0.0, rrt = 0.0, rtt = 0.0, ttt = 0.0, f_rr = 0.0, f_rt = 0.0, f_tt = 0.0;
+    auto add = [&](double g, double a, double b) {
+        const double ga = g * a, gb = g * b, gaa = ga * a, gab = ga * b, gbb = gb * b, s2 = fma(a, a, b * b);
+        rr = fma(ga, a, rr);
+        rt = fma(ga, b, rt);
+        tt = fma(gb, b, tt);
+        rrr = fma(gaa, a, rrr);
+        rrt = fma(gaa, b, rrt);
+        rtt = fma(gbb, a, rtt);
+        ttt = fma(gbb, b, ttt);
+        f_rr = fma(s2, gaa, f_rr);
+        f_rt = fma(s2, gab, f_rt);
+        f_tt = fma(s2, gbb, f_tt);
+    };
+    add(widen(fp[0]), -U, -V);
+#pragma unroll 1
+    for (int k = 0; k < 4; ++k) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            add(widen(fp[(1 + 8 * k + i) * plane]), fma(v[k], ex[i], -U), fma(v[k], ey[i], -V));
+            add(widen(fp[(5 + 8 * k + i) * plane]), fma(-v[k], ex[i], -U), fma(-v[k], ey[i], -V));
+        }
+    }
+    const double rT = 0.5 * (rr + tt), rTT2 = 2.0 * rT * (rT * inv_rho);
+    out[0] = rr - rT;
+    out[N] = rt;
+    out[2 * N] = tt - rT;
+    out[3 * N] = rrr;
+    out[4 * N] = rrt;
+    out[5 * N] = rtt;
+    out[6 * N] = ttt;
+    out[7 * N] = 0.5 * (rrr + rtt);
+    out[8 * N] = 0.5 * (rrt + ttt);
+    out[9 * N] = fma(0.5, f_rr, -rTT2);
+    out[10 * N] = 0.5 * f_rt;
+    out[11 * N] = fma(0.5, f_tt, -rTT2);
+}
+
 template <typename real>
 __global__ void __launch_bounds__(256) noneq_kernel(const MomArgs<real> A)
 {
@@ -1705,35 +1759,40 @@ __global__ void __launch_bounds__(256) noneq_kernel(const MomArgs<real> A)
             // M*_2 (central): rr, r-theta, theta-theta
             const double rr = fma(-rho, UU, 0.5 * (E2 + X2)), rt = fma(-rho, UV, 0.5 * Y2),
                          tt = fma(-rho, VV, 0.5 * (E2 - X2));
-            // M*_3: raw third moment less u's products with M*_2 and rho u u u
-            const double c3 = fma(rho, UU, 3.0 * rr), d3 = fma(rho, VV, 3.0 * tt);
-            const double rrr = fma(-U, c3, 0.25 * fma(3.0, A1, A3));
-            const double ttt = fma(-V, d3, 0.25 * fma(3.0, B1, -B3));
-            const double rrt = fma(-V, fma(rho, UU, rr), fma(-2.0 * U, rt, 0.25 * (B1 + B3)));
-            const double rtt = fma(-U, fma(rho, VV, tt), fma(-2.0 * V, rt, 0.25 * (A1 - A3)));
-            const double q_r = rrr + rtt, q_t = rrt + ttt;  // sum f |v*|^2 v*
-            // 2 M*_{4,2}: sum f |v|^2 v v less what u contributes
-            const double tr = rr + tt, w_r = fma(U, rr, V * rt), w_t = fma(U, rt, V * tt);
-            const double z = fma(rho, u2, tr);
-            const double h_r = q_r + 2.0 * w_r, h_t = q_t + 2.0 * w_t;
-            const double f_rr = fma(-UU, z, 0.5 * (E4 + X4)) - 2.0 * fma(U, h_r, fma(U, rrr, V * rrt)) - u2 * rr;
-            const double f_tt = fma(-VV, z, 0.5 * (E4 - X4)) - 2.0 * fma(V, h_t, fma(U, rtt, V * ttt)) - u2 * tt;
-            const double f_rt = fma(-UV, z, 0.5 * Y4) - fma(V, h_r, U * h_t) - 2.0 * fma(U, rrt, V * rtt) - u2 * rt;
-            // less the Maxwellian's: rho T = half the trace, 2 rho T^2
-            const double rT = 0.5 * tr, rTT2 = 2.0 * rT * (rT * inv_rho);
             double *out = A.out + s;
-            out[0] = rr - rT;
-            out[N] = rt;
-            out[2 * N] = tt - rT;
-            out[3 * N] = rrr;
-            out[4 * N] = rrt;
-            out[5 * N] = rtt;
-            out[6 * N] = ttt;
-            out[7 * N] = 0.5 * q_r;
-            out[8 * N] = 0.5 * q_t;
-            out[9 * N] = fma(0.5, f_rr, -rTT2);
-            out[10 * N] = 0.5 * f_rt;
-            out[11 * N] = fma(0.5, f_tt, -rTT2);
+            // u^2 > T / 4, rho u^2 against an eighth of 2 rho T by their upper words
+            if (sizeof(real) == 8 && __double2hiint(rho * u2) > __double2hiint(rr + tt) - (3 << 20)) {
+                central_sums(fp, A.plane, A.v, U, V, t, inv_rho, out, N);
+            } else {
+                // M*_3: raw third moment less u's products with M*_2 and rho u u u
+                const double c3 = fma(rho, UU, 3.0 * rr), d3 = fma(rho, VV, 3.0 * tt);
+                const double rrr = fma(-U, c3, 0.25 * fma(3.0, A1, A3));
+                const double ttt = fma(-V, d3, 0.25 * fma(3.0, B1, -B3));
+                const double rrt = fma(-V, fma(rho, UU, rr), fma(-2.0 * U, rt, 0.25 * (B1 + B3)));
+                const double rtt = fma(-U, fma(rho, VV, tt), fma(-2.0 * V, rt, 0.25 * (A1 - A3)));
+                const double q_r = rrr + rtt, q_t = rrt + ttt;  // sum f |v*|^2 v*
+                // 2 M*_{4,2}: sum f |v|^2 v v less what u contributes
+                const double tr = rr + tt, w_r = fma(U, rr, V * rt), w_t = fma(U, rt, V * tt);
+                const double z = fma(rho, u2, tr);
+                const double h_r = q_r + 2.0 * w_r, h_t = q_t + 2.0 * w_t;
+                const double f_rr = fma(-UU, z, 0.5 * (E4 + X4)) - 2.0 * fma(U, h_r, fma(U, rrr, V * rrt)) - u2 * rr;
+                const double f_tt = fma(-VV, z, 0.5 * (E4 - X4)) - 2.0 * fma(V, h_t, fma(U, rtt, V * ttt)) - u2 * tt;
+                const double f_rt = fma(-UV, z, 0.5 * Y4) - fma(V, h_r, U * h_t) - 2.0 * fma(U, rrt, V * rtt) - u2 * rt;
+                // less the Maxwellian's: rho T = half the trace, 2 rho T^2
+                const double rT = 0.5 * tr, rTT2 = 2.0 * rT * (rT * inv_rho);
+                out[0] = rr - rT;
+                out[N] = rt;
+                out[2 * N] = tt - rT;
+                out[3 * N] = rrr;
+                out[4 * N] = rrt;
+                out[5 * N] = rtt;
+                out[6 * N] = ttt;
+                out[7 * N] = 0.5 * q_r;
+                out[8 * N] = 0.5 * q_t;
+                out[9 * N] = fma(0.5, f_rr, -rTT2);
+                out[10 * N] = 0.5 * f_rt;
+                out[11 * N] = fma(0.5, f_tt, -rTT2);
+            }
         }
         __syncthreads();
     }

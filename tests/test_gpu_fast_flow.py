@@ -71,3 +71,40 @@ def test_temperature_is_as_exact_as_a_second_pass(u):
            for T in (got, _temperature(f, np.float64))]
     print("RMS", u, rms)
     assert rms[0] <= rms[1], rms
+
+
+def _delta(f, theta, real):
+    """Delta* by sums over v - u in the polar frame."""
+    f, rho, dx, dy = _about_u(f, real)
+    c, s = np.cos(theta.astype(np.longdouble)).astype(real), np.sin(theta.astype(np.longdouble)).astype(real)
+    a, b = dx * c[:, None] + dy * s[:, None], -dx * s[:, None] + dy * c[:, None]
+    M = [rho * 0 for _ in range(12)]
+    for q in range(33):
+        x, y, g = a[q], b[q], f[q]
+        h = g * (x * x + y * y) / 2
+        for k, term in enumerate((g * x * x, g * x * y, g * y * y, g * x * x * x, g * x * x * y, g * x * y * y,
+                                  g * y * y * y, h * x, h * y, h * x * x, h * x * y, h * y * y)):
+            M[k] = M[k] + term
+    T = (M[0] + M[2]) / (2 * rho)
+    for k, e in ((0, rho * T), (2, rho * T), (9, 2 * rho * T * T), (11, 2 * rho * T * T)):
+        M[k] = M[k] - e
+    return np.array(M)
+
+
+ORDERS = {"2": (0, 1, 2), "3": (3, 4, 5, 6), "3,1": (7, 8), "4,2": (9, 10, 11)}
+
+
+@pytest.mark.parametrize("u", [0.0, 0.5, 0.7, 1.0, 1.5, 2.0, 2.5])
+def test_delta_is_as_exact_as_central_sums(u):
+    from paper_1308_0653_gb300 import dbm
+    w, f, lam = _state(u)
+    sim = dbm.Simulation(dict(w.params, precision="fp64"))
+    sim.import_state(f, lam, 0)
+    got = sim.noneq()
+    sim.close()
+    theta = 2 * np.arctan2(np.longdouble(0), np.longdouble(-1)) * np.arange(f.shape[1]) / f.shape[1]
+    exact, plain = _delta(f, theta, np.longdouble), _delta(f, theta, np.float64)
+    rms = {k: [float(np.sqrt(np.mean((x[list(c)] - exact[list(c)]).astype(np.float64) ** 2))) for x in (got, plain)]
+           for k, c in ORDERS.items()}
+    print("RMS", u, rms)
+    assert all(a <= b for a, b in rms.values()), rms
