@@ -273,6 +273,9 @@ int dbm_launch_info(const dbm_t *h, int *grid, int *threads, int *smem_bytes,
  * device floats d_x into d_approx and d_ieee (device arrays); asynchronous. */
 int dbm_selftest_rcp(const float *d_x, float *d_approx, float *d_ieee, int n, void *stream);
 
+/* The same for the FP64 step's reciprocal (two Newton-Raphson steps). */
+int dbm_selftest_rcp64(const double *d_x, double *d_fast, double *d_ieee, int n, void *stream);
+
 /* Self-test of the bounded wait that every device-side wait of the step
  * kernels uses (an mbarrier wait that gives up after a cycle limit, sets a
  * status bit and returns instead of hanging).  One CTA waits on an mbarrier

@@ -1220,6 +1220,14 @@ int dbm_selftest_rcp(const float *d_x, float *d_approx, float *d_ieee, int n, vo
     return DBM_OK;
 }
 
+int dbm_selftest_rcp64(const double *d_x, double *d_fast, double *d_ieee, int n, void *stream)
+{
+    if (!d_x || !d_fast || !d_ieee || n < 0) return DBM_EINVAL;
+    cudaError_t e = launch_rcp64_selftest(d_x, d_fast, d_ieee, n, static_cast<cudaStream_t>(stream));
+    if (e != cudaSuccess) return cuda_fail(e, "FP64 rcp self-test launch");
+    return DBM_OK;
+}
+
 int dbm_selftest_wait(int *d_status, int arrive, int64_t limit_cycles, void *stream)
 {
     if (!d_status || limit_cycles < 1 || limit_cycles > kWaitLimitCycles) return DBM_EINVAL;

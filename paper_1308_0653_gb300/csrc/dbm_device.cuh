@@ -1317,6 +1317,15 @@ static __global__ void rcp_selftest_kernel(const float *x, float *approx, float 
     }
 }
 
+// Self-test of rcp64 against the correctly rounded division.
+static __global__ void rcp64_selftest_kernel(const double *x, double *fast, double *ieee, int n)
+{
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        fast[i] = rcp64(x[i]);
+        ieee[i] = __ddiv_rn(1.0, x[i]);
+    }
+}
+
 // ---------------------------------------------------------------------------
 // Initial state: f = f^eq(rho, u, T) (Eq. feq) of the initial fields, lambda
 // stored.  fields: [5][ntheta][nr] doubles (rho, u_r, u_theta, T, lambda).

@@ -21,6 +21,12 @@ cudaError_t launch_batch_direct64(const BatchArgs<double> &B, int nsm, int block
     return cudaGetLastError();
 }
 
+cudaError_t launch_rcp64_selftest(const double *x, double *fast, double *ieee, int n, cudaStream_t s)
+{
+    rcp64_selftest_kernel<<<256, 256, 0, s>>>(x, fast, ieee, n);
+    return cudaGetLastError();
+}
+
 cudaError_t batch_direct64_blocks(int *blocks_per_sm)
 {
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, (void *)batch_direct64_kernel<double>, 128, 0);

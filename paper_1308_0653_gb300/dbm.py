@@ -90,6 +90,7 @@ def lib():
         L.dbm_launch_info.argtypes = [H] + [ctypes.POINTER(ctypes.c_int)] * 6
         L.dbm_noneq.argtypes = [H, _dp, vp]
         L.dbm_noneq_device.argtypes = [H, vp, vp]
+        L.dbm_selftest_rcp64.argtypes = [vp, vp, vp, ctypes.c_int, vp]
         L.dbm_selftest_wait.argtypes = [vp, ctypes.c_int, ctypes.c_int64, vp]
         L.dbm_selftest_stop_loads.argtypes = [H, ctypes.c_int]
         L.dbm_num_variants.argtypes = [ctypes.c_int]
