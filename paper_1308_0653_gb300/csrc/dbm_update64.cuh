@@ -169,9 +169,11 @@ __device__ __forceinline__ void site_update64(const StepConsts<double> &C, const
     const double w[4] = {wx, H * Op64::add(wx, wy), wy, H * Op64::sub(wy, wx)};
 
     // Cochran rate with ignition gate, exact lambda step.  Below the gate a =
-    // b = 0, so R is 0, or NaN where lambda is not finite.
+    // b = 0, so the explicit R is 0, or NaN where lambda is not finite, and the
+    // consistent one, dlam / dt, is 0.
     double dlam = 0.0;
-    double R = (((uint32_t)__double2hiint(lam) >> 20) & 0x7ffu) == 0x7ffu ? lam - lam : 0.0;
+    const bool no_rate = (((uint32_t)__double2hiint(lam) >> 20) & 0x7ffu) == 0x7ffu && !C.reaction_energy;
+    double R = no_rate ? lam - lam : 0.0;
     const bool burns = T > C.T_th;
     if (__any_sync(ALL, burns)) {
         double a = 0.0, b = 0.0;
