@@ -294,6 +294,15 @@ int dbm_selftest_wait(int *d_status, int arrive, int64_t limit_cycles, void *str
  * the state undefined. */
 int dbm_selftest_stop_loads(dbm_t *h, int rows);
 
+/* The kernel that steps a simulation, or that a batch's last commit chose: the
+ * row ring, the one straight from global memory, or the one of single theta rows
+ * (-1: null handle).  dbm_launch_info and dbm_batch_launch_info report the row
+ * ring's shape whichever it is. */
+#define DBM_PATH_RING 0
+#define DBM_PATH_DIRECT 1
+#define DBM_PATH_ROW 2
+int dbm_step_path(const dbm_t *h);
+
 /* Number of step-kernel variants for a precision (0 if invalid).  Variants
  * differ only in how the work is staged (pipeline, ring depth, registers);
  * every variant computes the same update bit for bit. */
@@ -458,6 +467,9 @@ int dbm_batch_autotune(dbm_batch_t *b, int steps, void *stream, int *variant, in
  * then those of the row ring.  Null outputs are skipped. */
 int dbm_batch_launch_info(const dbm_batch_t *b, int *grid, int *items, int *rows_per_item,
                           int *variant);
+
+/* DBM_PATH_* of the batch's last commit (-1: null handle). */
+int dbm_batch_path(const dbm_batch_t *b);
 
 /* ---- serving: continuous batching behind submit / poll ------------------ */
 /*

@@ -1212,6 +1212,12 @@ int dbm_launch_info(const dbm_t *h, int *grid, int *threads, int *smem_bytes, in
     return DBM_OK;
 }
 
+int dbm_step_path(const dbm_t *h)
+{
+    if (!h) return -1;
+    return h->path == PATH_RING ? DBM_PATH_RING : h->path == PATH_ROW32 ? DBM_PATH_ROW : DBM_PATH_DIRECT;
+}
+
 int dbm_selftest_rcp(const float *d_x, float *d_approx, float *d_ieee, int n, void *stream)
 {
     if (!d_x || !d_approx || !d_ieee || n < 0) return DBM_EINVAL;
@@ -1984,6 +1990,12 @@ int dbm_batch_autotune(dbm_batch_t *b, int steps, void *stream, int *variant, in
     if (variant) *variant = bestv;
     if (rows_per_item) *rows_per_item = bestr;
     return DBM_OK;
+}
+
+int dbm_batch_path(const dbm_batch_t *b)
+{
+    if (!b) return -1;
+    return b->precision == DBM_FP64 || b->path == BATCH_DIRECT ? DBM_PATH_DIRECT : DBM_PATH_RING;
 }
 
 int dbm_batch_launch_info(const dbm_batch_t *b, int *grid, int *items, int *rows_per_item,

@@ -21,6 +21,7 @@ DBM_ETIMEOUT, DBM_ENONFINITE, DBM_ECUDA, DBM_ECANCELLED, DBM_ENOTFOUND, DBM_EDEV
 DBM_FP32, DBM_FP64 = 0, 1
 DBM_BC_OUTFLOW, DBM_BC_CENTRE = 0, 1
 DBM_R_EXPLICIT, DBM_R_CONSISTENT = 0, 1
+PATHS = ("ring", "direct", "row")  # DBM_PATH_*: the kernel that steps
 
 _dp = ctypes.POINTER(ctypes.c_double)
 
@@ -93,6 +94,7 @@ def lib():
         L.dbm_selftest_rcp64.argtypes = [vp, vp, vp, ctypes.c_int, vp]
         L.dbm_selftest_wait.argtypes = [vp, ctypes.c_int, ctypes.c_int64, vp]
         L.dbm_selftest_stop_loads.argtypes = [H, ctypes.c_int]
+        L.dbm_step_path.argtypes = [H]
         L.dbm_num_variants.argtypes = [ctypes.c_int]
         L.dbm_set_variant.argtypes = [H, ctypes.c_int]
         L.dbm_autotune.argtypes = [H, ctypes.c_int, vp, ctypes.POINTER(ctypes.c_int),
@@ -100,6 +102,7 @@ def lib():
         B = ctypes.c_void_p
         L.dbm_batch_bytes.argtypes = [ctypes.c_int, ctypes.c_int64, ctypes.c_int]
         L.dbm_batch_bytes.restype = ctypes.c_size_t
+        L.dbm_batch_path.argtypes = [B]
         _ip = ctypes.POINTER(ctypes.c_int32)
         L.dbm_batch_plan.argtypes = [ctypes.c_int32, _ip, _ip, _ip, ctypes.c_int32, ctypes.c_int32,
                                      ctypes.c_int64, _ip, ctypes.POINTER(ctypes.c_int64)]
@@ -320,6 +323,14 @@ def dbm_selftest_wait(dev_status_ptr: int, arrive: bool, limit_cycles: int, stre
                                    _stream(stream)), "dbm_selftest_wait")
 
 
+def dbm_step_path(h) -> str:
+    return PATHS[lib().dbm_step_path(h)]
+
+
+def dbm_batch_path(b) -> str:
+    return PATHS[lib().dbm_batch_path(b)]
+
+
 def dbm_num_variants(precision: int) -> int:
     return int(lib().dbm_num_variants(int(precision)))
 
@@ -465,6 +476,9 @@ class Simulation:
     def launch_info(self) -> dict:
         return dbm_launch_info(self.h)
 
+    def step_path(self) -> str:
+        return dbm_step_path(self.h)
+
     def state_device(self):
         """(f address, lambda address, ld) of the current state on the device."""
         return dbm_state_device(self.h)
@@ -553,6 +567,9 @@ class Batch:
 
     def launch_info(self) -> dict:
         return dbm_batch_launch_info(self.b)
+
+    def step_path(self) -> str:
+        return dbm_batch_path(self.b)
 
     def autotune(self, steps: int = 64, stream=None):
         return dbm_batch_autotune(self.b, steps, stream)
