@@ -1353,7 +1353,6 @@ struct dbm_batch_s {
     int grid;
     int nsm;
     BatchPath path;           // FP32: how it steps (as of the last commit)
-    bool ring_only;           // while dbm_batch_autotune compares shapes of the row ring
     int blocks64;             // resident blocks per SM of the FP64 direct kernel
     cudaGraphExec_t graphs[BATCH_PATHS];  // GRAPH_STEPS batch steps + counter advance
 };
@@ -1562,8 +1561,7 @@ std::vector<PlanItem> balance_items(const std::vector<PlanItem> &items, int grid
 // 3113 tiles of two larger ones 25.1 -> 28.4.
 bool batch_direct32(const dbm_batch_t *b, int tiles)
 {
-    return b->precision == DBM_FP32 && !b->ring_only && b->variant == default_variant<float>() &&
-           tiles <= 16 * b->nsm;
+    return b->precision == DBM_FP32 && b->variant == default_variant<float>() && tiles <= 16 * b->nsm;
 }
 
 // The row ring's way to a slot's constants.  Through uniform registers up to 40 000
@@ -1941,19 +1939,21 @@ int dbm_batch_autotune(dbm_batch_t *b, int steps, void *stream, int *variant, in
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
     int rc = DBM_OK, bestv = 0, bestr = 0;
-    float bestms = 0.f;
-    b->ring_only = true;
+    const int rows0 = b->rows_per_item;
+    float bestms = 0.f, ms = 0.f;
+    bool no_items = false;  // this variant steps the batch without work items: timed once, its rows stay
     for (int c = 0; c < 8 && rc == DBM_OK; ++c) {
         const int v = vs[c / 4], r = rows[c % 4];
-        if (ms_per_step) ms_per_step[c] = 0.f;
-        if (c >= 4 && vfb == vdef) continue;
+        if (c % 4 == 0) no_items = false;
+        if (ms_per_step) ms_per_step[c] = no_items ? ms : 0.f;
+        if (no_items || (c >= 4 && vfb == vdef)) continue;
         b->forced_variant = v;
         b->rows_per_item = r;
         b->dirty = true;
         rc = dbm_batch_step(b, GRAPH_STEPS, stream);  // commit, graph capture, warm-up
         if (rc != DBM_OK) break;
         if (b->variant != v) continue;  // the tensor-map kernel is not usable for this batch
-        float ms = 0.f;
+        no_items = dbm_batch_path(b) == DBM_PATH_DIRECT;
         for (int rep = 0; rep < 2 && rc == DBM_OK; ++rep) {  // the better of two timings
             cudaEventRecord(e0, st);
             rc = dbm_batch_step(b, steps, stream);
@@ -1973,11 +1973,10 @@ int dbm_batch_autotune(dbm_batch_t *b, int steps, void *stream, int *variant, in
         if (ms_per_step) ms_per_step[c] = ms;
         if (bestv == 0 || ms < bestms) {
             bestv = v;
-            bestr = r;
+            bestr = no_items ? rows0 : r;
             bestms = ms;
         }
     }
-    b->ring_only = false;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (rc != DBM_OK) return rc;
