@@ -428,7 +428,15 @@ int build_graph(dbm_t *h)
     return DBM_OK;
 }
 
-// Size classes of the autotuner: precision x ceil(log2 nr) x ceil(log2 ntheta).
+// FP32 grids up to four waves of 16 warps per SM step straight from global memory.
+bool direct32_grid(const dbm_params &p, int nsm)
+{
+    return (long long)((p.nr + 31) / 32) * p.ntheta <= 64LL * nsm;
+}
+
+// Size classes of the autotuner: precision x ceil(log2 nr) x ceil(log2 ntheta), those
+// that FP32's line between the kernels cuts in two (777 x 501 is on the ring, 600 x
+// 300 is not) once for each side.
 std::mutex g_tune_mu;
 std::map<long long, int> g_tuned;
 
@@ -439,13 +447,11 @@ long long size_class(const dbm_params &p)
         while ((1LL << l) < x) ++l;
         return l;
     };
-    return ((long long)p.precision << 16) | ((long long)lg(p.nr) << 8) | lg(p.ntheta);
-}
-
-// FP32 grids up to four waves of 16 warps per SM step straight from global memory.
-bool direct32_grid(const dbm_params &p, int nsm)
-{
-    return (long long)((p.nr + 31) / 32) * p.ntheta <= 64LL * nsm;
+    int dev = 0, nsm = 0;
+    const bool ring = p.precision == DBM_FP32 && cudaGetDevice(&dev) == cudaSuccess &&
+                      cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
+                      !direct32_grid(p, nsm);
+    return ((long long)ring << 20) | ((long long)p.precision << 16) | ((long long)lg(p.nr) << 8) | lg(p.ntheta);
 }
 
 // Rows that the busiest CTA of an FP32 ring loads per step (0: not known).
