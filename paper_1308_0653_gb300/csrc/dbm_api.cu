@@ -472,16 +472,19 @@ long long ring_rows(const dbm_params &p, int variant, int nsm)
 // (777 x 501, 10 rows against 14, 23.1 -> 21.4 us per step, 512 x 768 20.7 -> 18.9;
 // at 9/12 600^2 19.4 against 19.0 but 1492 x 270 21.2 against 21.4).  Larger grids
 // wait for HBM, where it makes no difference (1024^2 49.1 against 49.8, 2048 x 512
-// 48.9 against 50.1).
+// 48.9 against 50.1), but for strips of one warp's sites: the two CTAs' staged rows
+// are computed by all four warps (2 x 20000 108 us per step, 87 without staging, 61
+// on variant 5; 33 x 12000 68, 72 and 51).
 int pick_ring32(const dbm_params &p)
 {
     const int two = default_variant<float>(), three = 5;
     int dev = 0, nsm = 0, l2 = 0;
-    if (p.rows_per_item > 0 || p.ntheta == 1 || cudaGetDevice(&dev) != cudaSuccess ||
+    if (p.ntheta == 1 || cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess || direct32_grid(p, nsm))
         return two;
-    if (2LL * 33 * sizeof(float) * padded_ld(p.nr) * p.ntheta > l2) return two;
+    if (2LL * 33 * sizeof(float) * padded_ld(p.nr) * p.ntheta > l2) return p.nr <= 32 ? three : two;
+    if (p.rows_per_item > 0) return two;
     const long long r2 = ring_rows(p, two, nsm), r3 = ring_rows(p, three, nsm);
     return r2 > 0 && r3 > 0 && 15 * r3 <= 11 * r2 ? three : two;
 }

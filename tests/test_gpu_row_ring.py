@@ -45,6 +45,19 @@ def test_fp32_pipelines(nr, nth, shape, rows):
         assert np.array_equal(got[0], ref[0]) and np.array_equal(got[1], ref[1]), variant
 
 
+@pytest.mark.parametrize("nr,nth,shape,rows,variant", [
+    (2, 20000, {}, 0, 5), (32, 17000, DISC, 16, 5), (32, 9730, {}, 16, 4), (33, 12000, {}, 0, 4)])
+def test_fp32_strips_of_one_warp(nr, nth, shape, rows, variant):
+    """Three CTAs per SM, which leave out warps without a site, beyond L2."""
+    from paper_1308_0653_gb300 import dbm
+    w = workload(nr, nth, **shape)
+    sim = dbm.Simulation(dict(w.params, precision="fp32", rows_per_item=rows))
+    assert sim.launch_info()["variant"] == variant
+    sim.close()
+    got, ref = (_run(w, "fp32", v, "ring", (1, 4), rows) for v in (0, 2))
+    assert np.array_equal(got[0], ref[0]) and np.array_equal(got[1], ref[1])
+
+
 @pytest.mark.parametrize("nr,nth,shape,rows", [
     (130, 48, {}, 1), (200, 33, {}, 7), (64, 40, DISC, 0), (65, 9, DISC_SECTOR, 2), (300, 301, {}, 4),
     (700, 500, {}, 9)])  # the last two: several items per CTA
