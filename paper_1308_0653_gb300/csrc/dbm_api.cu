@@ -531,9 +531,7 @@ void fill_direct64(dbm_t *h)
 Path pick_path(const dbm_t *h)
 {
     const dbm_params &p = h->p;
-    const long long warps = (long long)((p.nr + 31) / 32) * p.ntheta;
-    if (p.precision == DBM_FP64)
-        return h->variant == default_variant<double>() && warps <= (1 << 29) ? PATH_DIRECT64 : PATH_RING;
+    if (p.precision == DBM_FP64) return h->variant == default_variant<double>() ? PATH_DIRECT64 : PATH_RING;
     if (h->variant != default_variant<float>()) return PATH_RING;
     if (p.ntheta == 1) return PATH_ROW32;
     return direct32_grid(p, h->nsm) ? PATH_DIRECT32 : PATH_RING;
@@ -565,7 +563,8 @@ int configure_launch(dbm_t *h, int variant)
         fill_step_args<double>(h, h->a64);
     else
         fill_step_args<float>(h, h->a32);
-    if (ki.version == 3 && !h->tmap_ok) {  // tensor maps not encodable for this grid
+    const bool direct64 = p.precision == DBM_FP64 && variant == default_variant<double>();
+    if (ki.version == 3 && !direct64 && !h->tmap_ok) {  // tensor maps not encodable for this grid
         h->ki = old_ki;
         if (old_ki.W) {
             if (p.precision == DBM_FP64)
@@ -1405,8 +1404,8 @@ long long batch_items(const dbm_batch_t *b, int cap)
 
 // Rows per item of a batch that does not fill the persistent CTAs a few times
 // over: a step then takes the busiest CTA's rows, ceil(items / CTAs) (rows + 2),
-// so items are cut shorter where that makes this smaller (one 512^2 simulation:
-// 128 items of 16 rows leave 176 of 304 CTAs idle, 296 of 7 take half the time).
+// so items are cut shorter where that makes this smaller (one 640 x 620 simulation:
+// 195 items of 16 rows leave 109 of 304 CTAs idle and take 18 rows, 285 of 11 take 13).
 int batch_row_cap(const dbm_batch_t *b)
 {
     int longest = 1;

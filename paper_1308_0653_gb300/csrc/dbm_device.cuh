@@ -258,8 +258,6 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t by
         : "memory");
 }
 
-template <typename real> __device__ __forceinline__ real rcp_(real x) { return real(1) / x; }
-
 template <typename real> __device__ __forceinline__ real expm1_(real x);
 template <> __device__ __forceinline__ float expm1_<float>(float x) { return expm1f(x); }
 template <> __device__ __forceinline__ double expm1_<double>(double x) { return expm1(x); }

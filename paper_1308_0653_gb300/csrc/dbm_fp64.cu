@@ -1,17 +1,17 @@
 // FP64 kernels (ALU-bound on GB300).  Variants as in the FP32 unit:
 //   1  v1  64  5  no   2
-//   2  v2  64  5  no   2   (a single simulation runs the direct kernel instead)
+//   2  the direct kernel (dbm_direct64.cuh); as launch information, variant 4's shape
 //   3  v2  64  4       3
 //   4  v3  64  5  no   2   (tensor-map TMA)
 //   5  v3  64  4       3   (tensor-map TMA)
 #include "dbm.h"
 #define DBM_REAL double
-#define DBM_VARIANTS(X) X(1, 1, 64, 5, false, 2) X(2, 2, 64, 5, false, 2) X(3, 2, 64, 4, false, 3) \
+#define DBM_VARIANTS(X) X(1, 1, 64, 5, false, 2) X(2, 3, 64, 5, false, 2) X(3, 2, 64, 4, false, 3) \
     X(4, 3, 64, 5, false, 2) X(5, 3, 64, 4, false, 3)
 #define DBM_DEFAULT_VARIANT 2
 #define DBM_FALLBACK_VARIANT 2
 #define DBM_RING_BATCH 0  // batches run the direct kernel
-#define DBM_BATCH_CONST_SLOTS DBM_BATCH_CONST_FP64  // batch constant table entries (304 B each)
+#define DBM_BATCH_CONST_SLOTS DBM_BATCH_CONST_FP64  // batch constant table entries (464 B each)
 #include "dbm_launch_impl.cuh"
 
 namespace dbm {
