@@ -377,7 +377,7 @@ int launch_pass(dbm_t *h, int b, int64_t left, cudaStream_t s, int *took)
     *took = 1;
     switch (h->path) {
     case PATH_ROW32:
-        *took = (int)std::min<int64_t>(left, Row32::MAX_STEPS);
+        *took = Row32::pass_steps(left);
         e = launch_row32(h->a32[b], *took, s);
         break;
     case PATH_DIRECT32: e = launch_direct32(h->a32[b], h->nsm, s); break;
