@@ -44,8 +44,8 @@ FALLBACK_HBM_GBS = 6800.0
 # kernel and launch sources still hash to the value it was taken with.
 KERNEL_SOURCES = ("dbm_device.cuh", "dbm_launch.h", "dbm_launch_impl.cuh", "dbm_fp32.cu", "dbm_api.cu")
 TRAFFIC_CAPTURES = [  # profiles/step_kernel_fp32_v4_implosion2048_dram.md
-    {"variant": 4, "nr": 2048, "ntheta": 2048, "bytes": 1105265493,
-     "sources_sha256": "bdd051381a23082f4190497647b4570e17454e09f3f6b5838a8776a3eab2dce6"},
+    {"variant": 4, "nr": 2048, "ntheta": 2048, "bytes": 1103262379,
+     "sources_sha256": "719be3edb2b811d5a841536c17a367c3b2b131ef009c68a196dee531dc43d4e6"},
 ]
 
 
@@ -327,7 +327,7 @@ def run_ours(args):
     elapsed = e0.elapsed_time(e1) / 1e3
     mom = sim.moments(stream=stream, raise_nonfinite=False)
     finite = mom["status"] == dbm.DBM_OK
-    launch = sim.launch_info()
+    launch, path = sim.launch_info(), sim.step_path()
     elapsed_max, units = aggregate(elapsed, float(sites) * NV * args.steps,
                                    backend_device=dev if ws > 1 else None)
     value = units / elapsed_max / 1e9
@@ -337,12 +337,13 @@ def run_ours(args):
     alg_bytes = BYTES_PER_SITE["fp32"] * sites
     achieved = alg_bytes / per_launch / 1e9
     peak, peak_src = measured_peak()
-    kname = {1: "dbm::step_kernel<float,128,6> (v1, row barrier)",
-             2: "dbm::step_kernel_v2<float,128,6,false,2,false> (bulk copies)",
-             3: "dbm::step_kernel_v2<float,128,4,true,3,false> (bulk copies)",
-             4: "dbm::step_kernel_v2<float,128,6,false,2,true> (tensor-map TMA)",
-             5: "dbm::step_kernel_v2<float,128,4,true,3,true> (tensor-map TMA)"}.get(
-                 launch["variant"], f"variant {launch['variant']}")
+    kname = {"direct": "dbm::direct32_kernel", "row": "dbm::row32_kernel"}.get(path) or {
+        1: "dbm::step_kernel<float,128,6> (v1, row barrier)",
+        2: "dbm::step_kernel_v2<float,128,6,false,2,false> (bulk copies)",
+        3: "dbm::step_kernel_v2<float,128,4,false,3,false> (bulk copies)",
+        4: "dbm::step_kernel_v2<float,128,5,true,2,true> (tensor-map TMA, staged row stores)",
+        5: "dbm::step_kernel_v2<float,128,4,false,3,true> (tensor-map TMA)"}.get(
+            launch["variant"], f"variant {launch['variant']}")
     roof = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
             "frac": achieved / peak, "traffic": measured_traffic(launch["variant"], w.params["nr"],
                                                                  w.params["ntheta"]),

@@ -86,7 +86,7 @@ typedef struct dbm_params {
     int32_t reaction_energy;   /* DBM_R_EXPLICIT (default) or DBM_R_CONSISTENT     */
     int32_t r_bc_inner;        /* DBM_BC_OUTFLOW or DBM_BC_CENTRE (r_in = 0)      */
     int32_t r_bc_outer;        /* DBM_BC_OUTFLOW                                  */
-    int32_t rows_per_item;     /* theta rows per CTA work item; 0 = automatic     */
+    int32_t rows_per_item;     /* theta rows per CTA work item of the row ring; 0 = automatic */
     int32_t variant;           /* step-kernel variant 1..dbm_num_variants();      */
                                /* 0 = autotuned choice for the size class, else   */
                                /* the library default                             */
@@ -440,7 +440,8 @@ int64_t dbm_batch_time(const dbm_batch_t *b);
  * precision's default (tensor-map row loads for FP32) when every attached
  * simulation has usable tensor maps, else the bulk-copy variant.  A change of
  * kernel waits for `stream` to drain and drops the captured step graph.
- * Errors: DBM_ENOMEM (more items than max_items), DBM_ECUDA. */
+ * Errors: DBM_ENOMEM (more items than max_items, counted for every kernel that
+ * may step the batch), DBM_ECUDA. */
 int dbm_batch_commit(dbm_batch_t *b, void *stream);
 
 /* Advance the step counter nsteps steps on `stream` (asynchronous); every
@@ -561,7 +562,8 @@ int dbm_submit(dbm_server_t *s, const dbm_params *p, const dbm_fields *init, int
  * still queued or running), DBM_ETIMEOUT, DBM_ENOTFOUND. */
 int dbm_poll(dbm_server_t *s, uint64_t ticket, dbm_result *out, int64_t timeout_us);
 
-/* Free the host arrays of a polled result. */
+/* Free the host arrays of a polled result (one block, which held the request's
+ * initial fields until then). */
 int dbm_result_free(dbm_result *res);
 
 /* Cancel a queued or running request (its result status becomes
