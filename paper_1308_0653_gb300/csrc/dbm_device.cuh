@@ -1606,7 +1606,7 @@ __global__ void __launch_bounds__(MOMENT_THREADS) moments_kernel(const MomArgs<r
             const double u2 = fma(ux, ux, uy * uy);
             double T = 0.5 * fma(e2, inv_rho, -u2);
             // by the upper words, FP64 instructions being what this kernel costs: u^2 > 1.25 to 1.5 T
-            if (__double2hiint(u2) > __double2hiint(T) + 0x80000) T = peculiar_T(fp, A.plane, A.vr, ux, uy, inv_rho);
+            if (__double2hiint(u2) > __double2hiint(T) + 0x80000LL) T = peculiar_T(fp, A.plane, A.vr, ux, uy, inv_rho);
             const double cth = A.rowtab[(long long)m * 16], sth = -A.rowtab[(long long)m * 16 + 8];
             const double ur = fma(ux, cth, uy * sth), uth = fma(uy, cth, -(ux * sth));
             const double lam = LamStore<real>::to_lambda((double)A.lam[(long long)m * A.ld + j]);
@@ -1773,7 +1773,7 @@ __global__ void __launch_bounds__(256) noneq_kernel(const MomArgs<real> A)
                          tt = fma(-rho, VV, 0.5 * (E2 - X2));
             double *out = A.out + s;
             // u^2 > T / 4, rho u^2 against an eighth of 2 rho T by their upper words
-            if (sizeof(real) == 8 && __double2hiint(rho * u2) > __double2hiint(rr + tt) - (3 << 20)) {
+            if (sizeof(real) == 8 && __double2hiint(rho * u2) > __double2hiint(rr + tt) - (3LL << 20)) {
                 central_sums(fp, A.plane, A.v, U, V, t, inv_rho, out, N);
             } else {
                 // M*_3: raw third moment less u's products with M*_2 and rho u u u
